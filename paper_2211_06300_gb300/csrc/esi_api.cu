@@ -74,6 +74,27 @@ struct DevSmp {
     int nrec = 0;
 };
 
+// Point lists of the on-chip 2D loops, by (shot, tile) of the loop plan.
+struct LoopInjBuf {
+    DBuf ptr, inj, patch_ptr, patch_blk;
+};
+struct LoopSmpBuf {
+    DBuf ptr, smp;
+};
+
+// How a 2D context's time loops run on chip (fd2loop.h): nsb shots per launch, gx x gz tiles
+// per shot, one CTA per tile.  ok is false where the loops stay with the per-step kernel.
+struct LoopPlan {
+    bool ok = false;
+    int nsb = 0, gx = 0, gz = 0;             // shots per launch, tiles per shot
+    int lanes = 1, nc = 0;                   // compute threads (LoopArgs)
+    int istride = 0;
+    size_t smem = 0;
+    LoopInjBuf inj_src, inj_rec;
+    LoopSmpBuf smp_rec, smp_src;
+    DBuf sync, inbox;
+};
+
 }  // namespace
 
 struct esi_ctx {
@@ -90,6 +111,9 @@ struct esi_ctx {
     int ntx = 0, nty = 1, ntz = 0, nzc = 1, ntiles = 0;
     int dft_k = DFT_BLOCK;         // steps per blocked DTFT pass (dft_block_steps)
     DBuf cc, kz, ky, kx, src_pos;
+    DBuf ac;                       // alpha c (2D: the on-chip loops)
+    // sponge rows [0, spz[0]) and [spz[1], nz) and columns likewise, where kappa is not zero
+    int spz[2] = {0, 0}, spx[2] = {0, 0};
     DBuf dev_err;                  // sticky device error word (int)
     struct TMap {
         const void *base;
@@ -99,6 +123,11 @@ struct esi_ctx {
     std::vector<TMap> tmaps;       // TMA maps of state buffers and of c (by address and box)
     DevInj inj_src, inj_rec;
     DevSmp smp_rec, smp_src;
+    LoopPlan lp;                   // on-chip time loops (2D)
+    // of a shot group's context: the loops launch for 1 / sm_share of the SMs and take the
+    // parent's cut, so that a shot's sums do not depend on the grouping
+    int sm_share = 1;
+    const LoopPlan *like = nullptr;
     DBuf u0, u1, a0, a1;           // forward / adjoint state pairs [ns][sst]
     DBuf part, part2, part3, scal; // reduction partials, per-shot scalars
     long long pc_fallbacks = 0;    // learned-preconditioner breakdowns (diagonal restart)
@@ -607,10 +636,272 @@ esi_status setup_model(esi_ctx *ctx, const void *vel, bool first) {
             }
             return p;
         };
+        auto range = [](const std::vector<T> &p, int n, int *r) {   // kappa falls to the inside
+            for (r[0] = 0; r[0] < n && p[r[0]] != T(0);) ++r[0];
+            for (r[1] = n; r[1] > r[0] && p[r[1] - 1] != T(0);) --r[1];
+        };
+        range(prof(ctx->g.nz, true, ctx->g.nz), ctx->g.nz, ctx->spz);
+        range(prof(ctx->g.nx, true, ctx->px), ctx->g.nx, ctx->spx);
         CK(upload(ctx->kz, prof(ctx->g.nz, true, ctx->g.nz), ctx->st));
         CK(upload(ctx->ky, prof(ctx->g.ny, ctx->g.ndim == 3, ctx->g.ny), ctx->st));
         // padded to the x pitch (zeros) for 16-byte loads
         CK(upload(ctx->kx, prof(ctx->g.nx, true, ctx->px), ctx->st));
+    }
+    if (ctx->g.ndim == 2) {
+        CK(ctx->ac.ensure(ctx->sst * sizeof(T)));
+        CKL(launch_alpha_c<T>(ctx->cc.as<T>(), ctx->kz.as<T>(), ctx->kx.as<T>(), ctx->ac.as<T>(),
+                              ctx->g.nz, ctx->px, ctx->st));
+    }
+    return ESI_OK;
+}
+
+// ------------------------------------------------------------------ plan of the on-chip loops
+struct LoopCand {
+    int nsb, gx, gz;     // shots per launch, tiles per shot along x and z
+    int lanes, rpt, nc;  // compute threads: lanes per group along x, rows each, count
+    double cost;
+};
+
+// largest part when n is cut into `parts` ranges
+inline int loop_ceil(int n, int parts) { return (n + parts - 1) / parts; }
+
+// The thread layout of a tile of nbx x nbz blocks, and the estimated time (us) of one of its
+// steps beside the exchange: a row of cells of every thread takes its dependence chain (FP32
+// about 420 cycles, up to about three warps per SM sub-partition) or, in FP64, 20 operations per
+// warp on units of half a lane per clock.
+void loop_layout(LoopCand &c, int nbx, int nbz, int esz, double &us) {
+    const int ncu = esz == 8 ? 4 * nbx : nbx, rows = 4 * nbz;
+    const int most = LOOP_THREADS - LOOP_COMM;
+    us = 1e300;
+    for (int lanes = 32; lanes >= 1; lanes /= 2) {
+        if (lanes > 2 * ncu && lanes > 1) continue;
+        const int ngx = loop_ceil(ncu, lanes);
+        if (ngx * lanes > most) continue;
+        const int rpt = loop_ceil(rows, std::min(most / (ngx * lanes), rows));
+        int nseg = loop_ceil(rows, rpt);
+        while (nseg * ngx * lanes % 32) ++nseg;   // whole warps
+        if (nseg * ngx * lanes > most) continue;
+        const int warps = nseg * ngx * lanes / 32;
+        const double w = loop_ceil(warps, 4);
+        // lanes below a quarter (FP32) or half (FP64) warp: shared-memory conflicts
+        const double conf = lanes >= (esz == 8 ? 16 : 8) ? 1.0 : 1.15;
+        const double row = esz == 8 ? std::max(1280.0 * w, 1500.0) : std::max(130.0 * w, 420.0) * conf;
+        const double t = rpt * row / 1950.0;
+        if (t < us * (1 - 1e-9)) {
+            us = t;
+            c.lanes = lanes, c.rpt = rpt, c.nc = warps * 32;
+        }
+    }
+}
+
+// Rows per thread beyond which the per-step kernel (bound by L2 / HBM, not by one chain of
+// dependent instructions per row) is the faster one in FP32.  us per step, loop against
+// per-step kernel: 801 x 241, 1 shot (1 row) 1.9 / 3.1 forward, 2.8 / 3.6 CG halves; 2 shots
+// (2 rows) 2.7 / 3.9 and 3.3 / 3.9; 3 shots (3 rows) 3.7 / 4.4 and 4.5 / 4.7; 4 shots (4 rows)
+// 4.3 / 4.7 and 5.3 / 4.9; 16 shots 10 / 9.8 and 16 / 13.7.  In FP64 the loop wins throughout (801 x
+// 241: 1 shot 11.7 / 23.1, 4 shots 38 / 77): whole warps on every SM's FP64 units.
+constexpr int LOOP_MAX_ROWS_F32 = 2;
+
+// estimated time of one step of every shot: launches x (exchange + the tile's rows + its rim)
+LoopCand loop_cost(int ns, int nsb, int gx, int gz, int qx, int gr, int esz) {
+    LoopCand c{nsb, gx, gz, 1, 1, 32, 0.0};
+    const int nbx = loop_ceil(qx, gx), nbz = loop_ceil(gr, gz);
+    const double rim = (gz > 1 ? nbx * (gz > 2 ? 2.0 : 1.0) : 0.0) + (gx > 1 ? nbz * (gx > 2 ? 2.0 : 1.0) : 0.0);
+    double us;
+    loop_layout(c, nbx, nbz, esz, us);
+    c.cost = loop_ceil(ns, nsb) * (0.8 + us + 0.004 * rim);
+    return c;
+}
+
+using InjShots = std::vector<std::vector<std::pair<HostPoint, Contrib>>>;
+
+// tile of a cell under a plan's cut, and the cell's place in it
+struct LoopTile {
+    int tile, q0, r0, nbx, nbz;
+};
+inline LoopTile loop_tile(const LoopCand &c, int qx, int gr, int iz, int ix) {
+    const int q = ix / 4, r = iz / 4;
+    int tx = (int)((long long)q * c.gx / qx), tz = (int)((long long)r * c.gz / gr);
+    while (tx + 1 < c.gx && loop_part(tx + 1, c.gx, qx) <= q) ++tx;
+    while (tz + 1 < c.gz && loop_part(tz + 1, c.gz, gr) <= r) ++tz;
+    LoopTile t;
+    t.tile = tz * c.gx + tx;
+    t.q0 = loop_part(tx, c.gx, qx);
+    t.r0 = loop_part(tz, c.gz, gr);
+    t.nbx = loop_part(tx + 1, c.gx, qx) - t.q0;
+    t.nbz = loop_part(tz + 1, c.gz, gr) - t.r0;
+    return t;
+}
+
+// host form of one injection list; bytes[tile] += its shared-memory tables
+template <typename T>
+struct LoopInjHost {
+    std::vector<int> ptr, patch_ptr, patch_blk;
+    std::vector<LoopInj<T>> inj;
+    void build(const LoopCand &c, int ns, int qx, int gr, const InjShots &shots, std::vector<size_t> &bytes) {
+        const int tiles = c.gx * c.gz;
+        bytes.assign((size_t)ns * tiles, 0);
+        ptr.assign(1, 0);
+        patch_ptr.assign(1, 0);
+        struct Node {
+            int tile, blk, cell, order;
+            Contrib con;
+        };
+        std::vector<Node> nodes;
+        for (int s = 0; s < ns; ++s) {
+            nodes.clear();
+            for (const auto &pc : shots[s]) {
+                const HostPoint &hp = pc.first;
+                for (size_t k = 0; k < hp.node.size(); ++k) {
+                    const LoopTile t = loop_tile(c, qx, gr, hp.iz[k], hp.ix[k]);
+                    const int lz = hp.iz[k] - 4 * t.r0, lx = hp.ix[k] - 4 * t.q0;
+                    Contrib con = pc.second;
+                    con.w *= hp.w[k];
+                    nodes.push_back({t.tile, (lz / 4) * t.nbx + lx / 4, (lz & 3) * 4 + (lx & 3),
+                                     (int)nodes.size(), con});
+                }
+            }
+            std::sort(nodes.begin(), nodes.end(), [](const Node &a, const Node &b) {
+                if (a.tile != b.tile) return a.tile < b.tile;
+                if (a.blk != b.blk) return a.blk < b.blk;
+                if (a.cell != b.cell) return a.cell < b.cell;
+                return a.order < b.order;
+            });
+            size_t k = 0;
+            for (int t = 0; t < tiles; ++t) {
+                int blk = -1, cell = -1, np = 0;
+                const size_t i0 = inj.size();
+                for (; k < nodes.size() && nodes[k].tile == t; ++k) {
+                    const Node &n = nodes[k];
+                    if (n.blk != blk) {
+                        patch_blk.push_back(n.blk);
+                        blk = n.blk, cell = -1;
+                        ++np;
+                    }
+                    inj.push_back({n.con.off0, n.con.tstride, n.cell == cell ? -1 : (np - 1) * 16 + n.cell, T(n.con.w)});
+                    cell = n.cell;
+                }
+                ptr.push_back((int)inj.size());
+                patch_ptr.push_back((int)patch_blk.size());
+                bytes[(size_t)s * tiles + t] = 32 * sizeof(T) * np + sizeof(LoopInj<T>) * (inj.size() - i0);
+            }
+        }
+    }
+    cudaError_t up(LoopInjBuf &b, cudaStream_t st) {
+        cudaError_t e;
+        if ((e = upload(b.ptr, ptr, st)) != cudaSuccess || (e = upload(b.inj, inj, st)) != cudaSuccess ||
+            (e = upload(b.patch_ptr, patch_ptr, st)) != cudaSuccess)
+            return e;
+        return upload(b.patch_blk, patch_blk, st);
+    }
+};
+
+// host form of one sampling list; false when a point needs the corner cell between four tiles,
+// which no tile holds (the exchange has no corners)
+template <typename T>
+struct LoopSmpHost {
+    std::vector<int> ptr;
+    std::vector<LoopSmp<T>> smp;
+    bool build(const LoopCand &c, int ns, int qx, int gr, const std::vector<SmpHost> &recs) {
+        const int tiles = c.gx * c.gz;
+        std::vector<std::pair<int, LoopSmp<T>>> all;   // by (shot, tile)
+        for (const SmpHost &h : recs) {
+            const LoopTile t = loop_tile(c, qx, gr, h.iz0, h.ix0);
+            const int P = 4 * t.nbx + 8;
+            LoopSmp<T> m{};
+            m.off = h.off0;
+            m.stride = h.tstride;
+            for (int j = 0; j < 4; ++j) {
+                const bool has = j < (int)h.hp.node.size();
+                const int lz = (has ? h.hp.iz[j] : h.iz0) - 4 * t.r0, lx = (has ? h.hp.ix[j] : h.ix0) - 4 * t.q0;
+                if (lz >= 4 * t.nbz && lx >= 4 * t.nbx) return false;
+                m.idx[j] = (lz + 4) * P + lx + 4;
+                m.w[j] = has ? T(h.hp.w[j] * h.scale) : T(0);
+            }
+            all.push_back({h.s * tiles + t.tile, m});
+        }
+        std::stable_sort(all.begin(), all.end(),
+                         [](const auto &a, const auto &b) { return a.first < b.first; });
+        ptr.assign((size_t)ns * tiles + 1, 0);
+        for (const auto &x : all) {
+            ++ptr[x.first + 1];
+            smp.push_back(x.second);
+        }
+        for (size_t i = 1; i < ptr.size(); ++i) ptr[i] += ptr[i - 1];
+        return true;
+    }
+    cudaError_t up(LoopSmpBuf &b, cudaStream_t st) {
+        cudaError_t e = upload(b.ptr, ptr, st);
+        return e != cudaSuccess ? e : upload(b.smp, smp, st);
+    }
+};
+
+// Chooses the cut of the on-chip loops: the cheapest whose tiles, with their point lists, fit in
+// shared memory and whose shots fit on the SMs; none (per-step kernel) when not even one shot
+// fits on the chip.
+template <typename T>
+esi_status setup_loops(esi_ctx *ctx, const InjShots &src_inj, const InjShots &rec_inj,
+                       const std::vector<SmpHost> &rec_smp, const std::vector<SmpHost> &src_smp) {
+    LoopPlan &lp = ctx->lp;
+    lp.ok = false;
+    if (ctx->g.ndim != 2) return ESI_OK;
+    int dev = 0, nsm = 0, coop = 0;
+    CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    CK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+    const int M = nsm;
+    if (!coop || M < 1 || (ctx->like && !ctx->like->ok)) return ESI_OK;
+    const int ns = ctx->ns, qx = (ctx->g.nx + 3) / 4, gr = (ctx->g.nz + 3) / 4;
+    auto tile_bytes = [&](const LoopCand &c) {
+        const size_t cols = 4 * (size_t)loop_ceil(qx, c.gx), rows = 4 * (size_t)loop_ceil(gr, c.gz);
+        // sponge corners: all sponge rows x columns (whole blocks) a tile can hold
+        const size_t cz = std::min(rows, (size_t)(ctx->spz[0] + ctx->g.nz - ctx->spz[1]));
+        const size_t cx = std::min(cols, (size_t)(ctx->spx[0] + ctx->g.nx - ctx->spx[1]) + 12);
+        return sizeof(T) * (2 * (cols + 8) * (rows + 8) + cols + rows + cz * cx) + cols * rows / 8 + 64;
+    };
+    std::vector<LoopCand> cand;
+    if (const LoopPlan *l = ctx->like)
+        cand.push_back({std::max(1, std::min(ns, M / ctx->sm_share / (l->gx * l->gz))), l->gx, l->gz, l->lanes, 0, l->nc, 0.0});
+    for (int nsb = ctx->like ? ns + 1 : 1; nsb <= std::min(ns, M); ++nsb) {
+        if (nsb > 1 && loop_ceil(ns, nsb) == loop_ceil(ns, nsb - 1) && nsb < ns) continue;
+        for (int gx = 1; gx <= std::min(qx, M / nsb); ++gx)
+            for (int gz = 1; gz <= std::min(gr, M / nsb / gx); ++gz) {
+                const LoopCand c = loop_cost(ns, nsb, gx, gz, qx, gr, ctx->esz);
+                // in FP32 one launch holds every shot or none: batches would add up their exchanges
+                if (sizeof(T) == 4 && (nsb < ns || c.rpt > LOOP_MAX_ROWS_F32)) continue;
+                if (tile_bytes(c) <= (size_t)LOOP_SMEM) cand.push_back(c);
+            }
+    }
+    std::stable_sort(cand.begin(), cand.end(), [](const LoopCand &a, const LoopCand &b) { return a.cost < b.cost; });
+    for (size_t i = 0; i < cand.size() && i < 24; ++i) {
+        const LoopCand &c = cand[i];
+        LoopSmpHost<T> sr, ss;
+        if (!sr.build(c, ns, qx, gr, rec_smp) || !ss.build(c, ns, qx, gr, src_smp)) continue;
+        LoopInjHost<T> is, ir;
+        std::vector<size_t> bs, br;
+        is.build(c, ns, qx, gr, src_inj, bs);
+        ir.build(c, ns, qx, gr, rec_inj, br);
+        size_t lists = 0;
+        for (size_t k = 0; k < bs.size(); ++k) lists = std::max(lists, std::max(bs[k], br[k]));
+        if (tile_bytes(c) + lists > (size_t)LOOP_SMEM) continue;
+        const int nbx = loop_ceil(qx, c.gx), nbz = loop_ceil(gr, c.gz);
+        lp.nsb = c.nsb, lp.gx = c.gx, lp.gz = c.gz;
+        lp.lanes = c.lanes, lp.nc = c.nc;
+        lp.smem = tile_bytes(c) + lists;
+        const int epr = sizeof(T) == 4 ? 2 : 4;
+        lp.istride = 2 * (nbx + nbz) * 4 * epr;
+        const size_t ib = (size_t)2 * c.nsb * c.gx * c.gz * lp.istride * 16;
+        CK(lp.inbox.ensure(ib));
+        CK(lp.sync.ensure(16));
+        CK(cudaMemsetAsync(lp.inbox.p, 0, ib, ctx->st));
+        CK(cudaMemsetAsync(lp.sync.p, 0, 16, ctx->st));
+        CK(is.up(lp.inj_src, ctx->st));
+        CK(ir.up(lp.inj_rec, ctx->st));
+        CK(sr.up(lp.smp_rec, ctx->st));
+        CK(ss.up(lp.smp_src, ctx->st));
+        CK(cudaStreamSynchronize(ctx->st));   // the host lists end with this scope
+        lp.ok = true;
+        break;
     }
     return ESI_OK;
 }
@@ -645,6 +936,7 @@ esi_status setup_geometry(esi_ctx *ctx) {
     if ((e = build_inj<T>(ctx, ctx->inj_rec, rec_inj)) != ESI_OK) return e;
     if ((e = build_smp<T>(ctx, ctx->smp_rec, rec_smp)) != ESI_OK) return e;
     if ((e = build_smp<T>(ctx, ctx->smp_src, src_smp)) != ESI_OK) return e;
+    if ((e = setup_loops<T>(ctx, src_inj, rec_inj, rec_smp, src_smp)) != ESI_OK) return e;
     CK(upload(ctx->src_pos, ctx->src_xyz, ctx->st));
     return ESI_OK;
 }
@@ -750,6 +1042,55 @@ esi_status graph_capture(esi_ctx *ctx, std::vector<unsigned char> &&key, F &&bod
     return st;
 }
 
+// ------------------------------------------------------------------ on-chip loops (2D)
+// A run of fewer steps does not pay for reading and writing the states once around it.
+constexpr int LOOP_MIN_STEPS = 8;
+
+bool loop_ready(const esi_ctx *ctx, int steps) {
+    return ctx->g.ndim == 2 && ctx->lp.ok && steps >= LOOP_MIN_STEPS;
+}
+
+// `steps` time steps of variant `flags` on chip, every time index of `a` (given for the first
+// step) moving by dn; states as in the per-step loops: cur and po are read, and after the run
+// the newer state is in cur when steps is even, in po when it is odd.
+template <typename T>
+esi_status loop_run(esi_ctx *ctx, unsigned flags, StepArgs<T> a, T *cur, T *po, int steps, int dn) {
+    LoopPlan &lp = ctx->lp;
+    LoopArgs<T> g;
+    std::memset(&g, 0, sizeof(g));
+    a.cur = cur;
+    a.po = po;
+    g.gx = lp.gx, g.gz = lp.gz;
+    g.qx = (ctx->g.nx + 3) / 4, g.gr = (ctx->g.nz + 3) / 4;
+    g.steps = steps, g.dn = dn, g.nt = ctx->nt;
+    g.nc = lp.nc, g.nm = LOOP_COMM;
+    g.lanes = lp.lanes;
+    g.nbz0 = ctx->spz[0], g.nbz1 = ctx->spz[1], g.nbx0 = ctx->spx[0], g.nbx1 = ctx->spx[1];
+    g.ac = ctx->ac.as<T>();
+    g.sync = lp.sync.as<unsigned>();
+    g.inbox = lp.inbox.as<ulonglong2>();
+    g.istride = lp.istride;
+    g.dot_stride = lp.gx * lp.gz;
+    if (flags & F_PT) {
+        LoopInjBuf &l = a.inj.tile_ptr == ctx->inj_src.tile_ptr.as<int>() ? lp.inj_src : lp.inj_rec;
+        g.inj_ptr = l.ptr.as<int>();
+        g.inj = l.inj.as<LoopInj<T>>();
+        g.patch_ptr = l.patch_ptr.as<int>();
+        g.patch_blk = l.patch_blk.as<int>();
+    }
+    if (flags & F_SMP) {
+        LoopSmpBuf &l = a.smp.tile_ptr == ctx->smp_src.tile_ptr.as<int>() ? lp.smp_src : lp.smp_rec;
+        g.smp_ptr = l.ptr.as<int>();
+        g.smp = l.smp.as<LoopSmp<T>>();
+    }
+    for (int s0 = 0; s0 < ctx->ns; s0 += lp.nsb) {
+        g.s0 = s0;
+        const int nblk = std::min(lp.nsb, ctx->ns - s0) * lp.gx * lp.gz;
+        CKL(launch_loop2<T>(flags, a, g, nblk, lp.nc + LOOP_COMM, lp.smem, ctx->st));
+    }
+    return ESI_OK;
+}
+
 // ------------------------------------------------------------------ forward modelling
 // Runs steps [n0, n1) starting from states (cur, po) = (u_{n0}, u_{n0-1}); on return
 // cur holds u_{n1}.  Sampling of the inputs writes traces[n-1].
@@ -775,7 +1116,12 @@ esi_status fwd_loop(esi_ctx *ctx, StepArgs<T> a, unsigned flags, T *&cur, T *&po
         return ESI_OK;
     };
     esi_status e;
-    if (ctx->use_graphs && n1 - n0 >= GRAPH_MIN_STEPS) {
+    if (loop_ready(ctx, n1 - n0)) {
+        a.n = a.tin = n0;
+        a.tout = n0 - 1;
+        a.slot_w = 0;
+        e = loop_run<T>(ctx, flags, a, c0, p0, n1 - n0, +1);
+    } else if (ctx->use_graphs && n1 - n0 >= GRAPH_MIN_STEPS) {
         auto key = loop_key(a, flags, +1, n0, n1, false, c0, p0);
         if (!graph_replay(ctx, key, e)) e = graph_capture(ctx, std::move(key), body);
     } else {
@@ -799,7 +1145,14 @@ esi_status fwd_dft_loop(esi_ctx *ctx, StepArgs<T> a, unsigned flags, T *cur, T *
         T *c = cur, *q = po;
         for (int n0 = 0; n0 < nt; n0 += ctx->dft_k) {
             const int n1 = std::min(nt, n0 + ctx->dft_k);
-            for (int n = n0; n < n1; ++n) {
+            if (loop_ready(ctx, n1 - n0)) {
+                a.n = a.tin = n0;
+                a.tout = n0 - 1;
+                a.slot_w = 0;
+                esi_status e = loop_run<T>(ctx, flags, a, c, q, n1 - n0, +1);
+                if (e != ESI_OK) return e;
+                if ((n1 - n0) & 1) std::swap(c, q);
+            } else for (int n = n0; n < n1; ++n) {
                 a.cur = c;
                 a.po = q;
                 a.n = n;
@@ -817,7 +1170,7 @@ esi_status fwd_dft_loop(esi_ctx *ctx, StepArgs<T> a, unsigned flags, T *cur, T *
         return ESI_OK;
     };
     esi_status e;
-    if (ctx->use_graphs && nt >= GRAPH_MIN_STEPS) {
+    if (ctx->use_graphs && nt >= GRAPH_MIN_STEPS && !loop_ready(ctx, ctx->dft_k)) {
         auto key = loop_key(a, flags, +2, 0, nt, false, cur, po);
         if (!graph_replay(ctx, key, e)) e = graph_capture(ctx, std::move(key), body);
     } else {
@@ -989,7 +1342,12 @@ esi_status adj_loop(esi_ctx *ctx, StepArgs<T> a, unsigned flags, T *&cur, T *&po
         return ESI_OK;
     };
     esi_status e;
-    if (ctx->use_graphs && j1 - j0 >= GRAPH_MIN_STEPS) {
+    if (loop_ready(ctx, j1 - j0)) {
+        a.n = a.tin = a.nout = j1 - 1;
+        a.tout = j1;   // sampled while within the record
+        a.slot_r = j1 - 1 - j0;
+        e = loop_run<T>(ctx, flags, a, c0, p0, j1 - j0, -1);
+    } else if (ctx->use_graphs && j1 - j0 >= GRAPH_MIN_STEPS) {
         auto key = loop_key(a, flags, -1, j0, j1, sample_src, c0, p0);
         if (!graph_replay(ctx, key, e)) e = graph_capture(ctx, std::move(key), body);
     } else {
@@ -1317,9 +1675,11 @@ esi_status cg_impl(esi_ctx *ctx, double lambda, double tol, int max_iter, const 
     CK(ctx->cg_p.ensure(vb));
     CK(ctx->cg_ap.ensure(vb));
     CK(ctx->traces.ensure(std::max<size_t>((size_t)ctx->total_rec * nt * sizeof(T), 16)));
-    // <p, A p> partials of the adjoint half: one per warp of a 2D tile, one per 3D block
-    const int nblk_step = ctx->g.ndim == 2 ? ctx->ntx * ctx->ntz * (NT2 / 32)
-                                            : ctx->ntx * ctx->nty * ctx->nzc;
+    // <p, A p> partials per shot of the adjoint half: one per tile of the on-chip loop, one per
+    // warp of a 2D tile of the per-step kernel, one per 3D block
+    const int nblk_step = loop_ready(ctx, nt) ? ctx->lp.gx * ctx->lp.gz
+                          : ctx->g.ndim == 2  ? ctx->ntx * ctx->ntz * (NT2 / 32)
+                                              : ctx->ntx * ctx->nty * ctx->nzc;
     const int nblk_vec = 1216;  // 8 x 152 SMs
     const size_t npart = (size_t)ns * std::max(nblk_step, nblk_vec);
     CK(ctx->part.ensure(sizeof(double) * npart));
@@ -1889,7 +2249,14 @@ esi_status fdcg_impl(esi_ctx *ctx, double lambda, double tol, int max_iter, cons
             T *c = c0, *q = p0;
             for (int jhi = nt; jhi > 0;) {
                 const int jlo = std::max(0, jhi - K);
-                for (int j = jhi; j > jlo; --j) {
+                if (loop_ready(ctx, jhi - jlo)) {
+                    a.n = a.tin = a.nout = jhi - 1;
+                    a.tout = -1;
+                    a.slot_w = jhi - 1 - jlo;
+                    esi_status st = loop_run<T>(ctx, aflags, a, c, q, jhi - jlo, -1);
+                    if (st != ESI_OK) return st;
+                    if ((jhi - jlo) & 1) std::swap(c, q);
+                } else for (int j = jhi; j > jlo; --j) {
                     a.cur = c;
                     a.po = q;
                     a.n = j - 1;
@@ -1908,7 +2275,7 @@ esi_status fdcg_impl(esi_ctx *ctx, double lambda, double tol, int max_iter, cons
             return ESI_OK;
         };
         esi_status st;
-        if (ctx->use_graphs && nt >= GRAPH_MIN_STEPS) {
+        if (ctx->use_graphs && nt >= GRAPH_MIN_STEPS && !loop_ready(ctx, K)) {
             auto key = loop_key(a, aflags, -3, part, nt, false, c0, p0);
             if (!graph_replay(ctx, key, st)) st = graph_capture(ctx, std::move(key), body);
         } else {
@@ -1943,7 +2310,14 @@ esi_status fdcg_impl(esi_ctx *ctx, double lambda, double tol, int max_iter, cons
                 const int n1 = std::min(nt, n0 + K);
                 CKL(launch_idft_block<T>(qb, n1 - n0, K, ns, ctx->sst, nf,
                                          a.twid + (size_t)n0 * nf * 2, src, ctx->st));
-                for (int n = n0; n < n1; ++n) {
+                if (loop_ready(ctx, n1 - n0)) {
+                    a.n = 0;   // the stash slot
+                    a.tin = n0;
+                    a.tout = n0 - 1;
+                    esi_status st = loop_run<T>(ctx, F_CGP | F_SMP, a, c, q, n1 - n0, +1);
+                    if (st != ESI_OK) return st;
+                    if ((n1 - n0) & 1) std::swap(c, q);
+                } else for (int n = n0; n < n1; ++n) {
                     a.cur = c;
                     a.po = q;
                     a.n = n - n0;   // the stash slot
@@ -1958,7 +2332,7 @@ esi_status fdcg_impl(esi_ctx *ctx, double lambda, double tol, int max_iter, cons
             return ESI_OK;
         };
         esi_status st;
-        if (ctx->use_graphs && nt >= GRAPH_MIN_STEPS) {
+        if (ctx->use_graphs && nt >= GRAPH_MIN_STEPS && !loop_ready(ctx, K)) {
             auto key = loop_key(a, F_CGP | F_SMP, +3, part, nt, false, c0, p0);
             if (!graph_replay(ctx, key, st)) st = graph_capture(ctx, std::move(key), body);
         } else {
@@ -2517,8 +2891,10 @@ ESI_API int esi_get_profile(esi_ctx *ctx, esi_kernel_stat *out, int max) {
     return n;
 }
 
-ESI_API esi_status esi_create(esi_ctx **out, const esi_grid *grid, const esi_geometry *geom,
-                              const void *velocity_dev, double dt, int nt, void *stream) {
+namespace {
+esi_status create_ctx(esi_ctx **out, const esi_grid *grid, const esi_geometry *geom,
+                      const void *velocity_dev, double dt, int nt, void *stream, int sm_share,
+                      const LoopPlan *like) {
     g_create_error.clear();
     if (!out || !grid || !geom || !velocity_dev) return ESI_ERR_ARG;
     *out = nullptr;
@@ -2540,6 +2916,8 @@ ESI_API esi_status esi_create(esi_ctx **out, const esi_grid *grid, const esi_geo
     ctx->esz = g.dtype == ESI_F64 ? 8 : 4;
     ctx->N = (long long)g.nz * g.ny * g.nx;
     ctx->px = (g.nx + PITCH - 1) / PITCH * PITCH;
+    ctx->sm_share = sm_share;
+    ctx->like = like;
     ctx->sst = (long long)g.nz * g.ny * ctx->px;
     ctx->src_xyz.assign(geom->src_xyz, geom->src_xyz + 3 * geom->ns);
     ctx->rec_off.assign(geom->rec_offset, geom->rec_offset + geom->ns + 1);
@@ -2575,8 +2953,15 @@ ESI_API esi_status esi_create(esi_ctx **out, const esi_grid *grid, const esi_geo
         g_create_error = c->err;  // readable through esi_last_error(NULL)
         return e;
     }
+    c->like = nullptr;   // used at creation only
     *out = ctx.release();
     return ESI_OK;
+}
+}  // namespace
+
+ESI_API esi_status esi_create(esi_ctx **out, const esi_grid *grid, const esi_geometry *geom,
+                              const void *velocity_dev, double dt, int nt, void *stream) {
+    return create_ctx(out, grid, geom, velocity_dev, dt, nt, stream, 1, nullptr);
 }
 
 ESI_API void esi_destroy(esi_ctx *ctx) {
@@ -2621,7 +3006,7 @@ ESI_API esi_status esi_set_shot_groups(esi_ctx *ctx, int groups, const void *vel
         }
         ctx->grp_st.push_back(st);
         esi_ctx *c = nullptr;
-        const esi_status e = esi_create(&c, &g, &sub, velocity_dev, ctx->dt, ctx->nt, st);
+        const esi_status e = create_ctx(&c, &g, &sub, velocity_dev, ctx->dt, ctx->nt, st, groups, &ctx->lp);
         if (e != ESI_OK) {
             const std::string m = esi_last_error(nullptr);
             ctx->clear_groups();

@@ -165,6 +165,7 @@ struct StepArgs {
 
 // device error codes written to StepArgs::dev_err
 constexpr int DEV_ERR_TMA_TIMEOUT = 1;
+constexpr int DEV_ERR_LOOP_TIMEOUT = 2;
 // iteration limit of the mbarrier wait for a TMA tile (a tile arrives in microseconds;
 // the limit is seconds of polling)
 constexpr long long TMA_WAIT_LIMIT = 1ll << 26;
@@ -180,6 +181,61 @@ cudaError_t launch_step3(unsigned flags, const StepArgs<T> &a, int ns, cudaStrea
 // (the resident blocks per SM of the step kernel on the current device enter the choice)
 int step3_chunks(int nz, long long cols, int esz);
 
+// ----------------------------------------------------------------------------- on-chip loops
+// 2D time loops whose states stay in shared memory (fd2loop.h): the plane is cut into 4 x 4
+// cell blocks, a tile is a range of block columns x a range of block rows.
+constexpr int LOOP_THREADS = 512;        // compute + communication threads, at most
+constexpr int LOOP_COMM = 128;           // communication threads
+constexpr int LOOP_SMEM = 226 * 1024;    // dynamic shared memory of a tile, at most
+
+// first block of part i when n blocks are cut into `parts` near-equal ranges
+__host__ __device__ inline int loop_part(int i, int parts, int n) {
+    return (int)((long long)i * n / parts);
+}
+
+// one contribution to a point-source cell: value w * trace[off + t * stride]; pos = the cell's
+// place in the tile's patches (16 values per block), or -1 when it adds to the entry before it
+template <typename T>
+struct LoopInj {
+    long long off;
+    int stride, pos;
+    T w;
+};
+// one receiver: four points of the tile's shared-memory array, and its trace
+template <typename T>
+struct LoopSmp {
+    int idx[4];
+    T w[4];
+    long long off;
+    int stride;
+};
+
+template <typename T>
+struct LoopArgs {
+    int s0;                  // first shot of this launch
+    int gx, gz;              // tiles per shot along x and z
+    int qx, gr;              // block columns and block rows of the plane
+    int steps, dn;           // time steps; increment (+1 / -1) of every time index per step
+    int nt;                  // traces are sampled at 0 <= tout < nt
+    int nc, nm;              // compute and communication threads
+    int lanes;               // lanes along x per group of compute threads
+    int nbz0, nbz1, nbx0, nbx1;   // sponge rows: [0, nbz0) and [nbz1, nz); columns likewise
+    const T *ac;             // alpha c per cell (alpha = 1 / (1 + kappa)), pitched
+    unsigned *sync;          // [0] tag epoch, [1] finished CTAs
+    ulonglong2 *inbox;       // [parity][CTA][istride] packets from the neighbours
+    int istride;
+    int dot_stride;          // partials per shot in StepArgs::dot_part
+    // lists by (shot, tile)
+    const int *inj_ptr, *patch_ptr, *smp_ptr;
+    const LoopInj<T> *inj;
+    const int *patch_blk;    // blocks of the tile that hold point sources
+    const LoopSmp<T> *smp;
+};
+
+template <typename T>
+cudaError_t launch_loop2(unsigned flags, const StepArgs<T> &a, const LoopArgs<T> &g, int nblk,
+                         int threads, size_t smem, cudaStream_t st);
+
 // sample a whole state (global memory) for every receiver of a list at time tout
 template <typename T>
 cudaError_t launch_sample_global(const SmpList<T> &l, const T *state, long long sst, T *out,
@@ -189,6 +245,11 @@ cudaError_t launch_sample_global(const SmpList<T> &l, const T *state, long long 
 template <typename T>
 cudaError_t launch_setup_cc(const T *v, T *cc, int nz, int ny, int nx, int px, double dt,
                             double dx, double *vmax_part, int nblk, cudaStream_t st);
+
+// ac = alpha cc over the pitched 2D plane, alpha = 1 / (1 + kz + kx) (pad cells 0)
+template <typename T>
+cudaError_t launch_alpha_c(const T *cc, const T *kz, const T *kx, T *ac, int nz, int px,
+                           cudaStream_t st);
 
 // per-shot reductions of dense [ns][len] vectors into block partials [ns][nblk]
 template <typename T>

@@ -60,6 +60,19 @@ __global__ void setup_cc_kernel(const T *v, T *cc, int nz, int ny, int nx, int p
     }
 }
 
+// ac = alpha cc, the update's factor of S in the on-chip loops: the sponge's divisions once per
+// model instead of once per cell and step; the rounding of the step kernel's al * cc
+template <typename T>
+__global__ void alpha_c_kernel(const T *cc, const T *kz, const T *kx, T *ac, int nz, int px) {
+    const long long n = (long long)nz * px;
+    for (long long i = (long long)blockIdx.x * RT + threadIdx.x; i < n; i += (long long)gridDim.x * RT) {
+        const int z = int(i / px), x = int(i - (long long)z * px);
+        const T kap = kz[z] + kx[x];
+        const T al = T(1) / (T(1) + kap);
+        ac[i] = al * cc[i];
+    }
+}
+
 // <a, b> per shot over pitched vectors (len a multiple of the 16-byte vector width; pad
 // elements are zero): 16-byte loads, a field-precision sum per vector, double across.
 template <typename T>
@@ -582,6 +595,13 @@ template <typename T>
 cudaError_t launch_setup_cc(const T *v, T *cc, int nz, int ny, int nx, int px, double dt,
                             double dx, double *vmax_part, int nblk, cudaStream_t st) {
     setup_cc_kernel<T><<<nblk, RT, 0, st>>>(v, cc, nz, ny, nx, px, dt, dx, vmax_part);
+    return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_alpha_c(const T *cc, const T *kz, const T *kx, T *ac, int nz, int px,
+                           cudaStream_t st) {
+    alpha_c_kernel<T><<<blocks_for((long long)nz * px, 2048), RT, 0, st>>>(cc, kz, kx, ac, nz, px);
     return cudaGetLastError();
 }
 
@@ -1210,6 +1230,8 @@ cudaError_t launch_mlincomb(T *z, double alpha, const T *x, double beta, const T
 }
 
 #define ESI_INST(T)                                                                              \
+    template cudaError_t launch_alpha_c<T>(const T *, const T *, const T *, T *, int, int,       \
+                                           cudaStream_t);                                        \
     template cudaError_t launch_setup_cc<T>(const T *, T *, int, int, int, int, double, double,  \
                                             double *, int, cudaStream_t);                        \
     template cudaError_t launch_dot<T>(const T *, const T *, long long, long long, int, double *, \
