@@ -862,13 +862,14 @@ esi_status setup_loops(esi_ctx *ctx, const InjShots &src_inj, const InjShots &re
     std::vector<LoopCand> cand;
     if (const LoopPlan *l = ctx->like)
         cand.push_back({std::max(1, std::min(ns, M / ctx->sm_share / (l->gx * l->gz))), l->gx, l->gz, l->lanes, 0, l->nc, 0.0});
-    for (int nsb = ctx->like ? ns + 1 : 1; nsb <= std::min(ns, M); ++nsb) {
+    // in FP32 one launch holds every shot or none: batches would add up their exchanges
+    for (int nsb = ctx->like ? ns + 1 : sizeof(T) == 4 ? ns : 1; nsb <= std::min(ns, M); ++nsb) {
         if (nsb > 1 && loop_ceil(ns, nsb) == loop_ceil(ns, nsb - 1) && nsb < ns) continue;
         for (int gx = 1; gx <= std::min(qx, M / nsb); ++gx)
             for (int gz = 1; gz <= std::min(gr, M / nsb / gx); ++gz) {
                 const LoopCand c = loop_cost(ns, nsb, gx, gz, qx, gr, ctx->esz);
-                // in FP32 one launch holds every shot or none: batches would add up their exchanges
-                if (sizeof(T) == 4 && (nsb < ns || c.rpt > LOOP_MAX_ROWS_F32)) continue;
+                if (!(c.cost < 1e300)) continue;   // no layout of the threads covers such a tile
+                if (sizeof(T) == 4 && c.rpt > LOOP_MAX_ROWS_F32) continue;
                 if (tile_bytes(c) <= (size_t)LOOP_SMEM) cand.push_back(c);
             }
     }

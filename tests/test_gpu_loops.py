@@ -15,7 +15,9 @@ pytestmark = pytest.mark.gpu
 CASES = [  # nz, nx, shots, steps, sponge cells
     (5, 7, 1, 40, 1), (9, 300, 2, 40, 2), (300, 9, 2, 40, 2), (45, 83, 3, 90, 6),
     (101, 101, 1, 120, 20), (241, 801, 1, 60, 20), (241, 801, 16, 40, 20),
-    (301, 1201, 9, 24, 20), (64, 1600, 3, 30, 8), (97, 130, 40, 33, 8), (45, 83, 3, 8, 6)]
+    (301, 1201, 9, 24, 20), (64, 1600, 3, 30, 8), (97, 130, 40, 33, 8), (45, 83, 3, 8, 6),
+    # tiles of the whole width fit the shared memory, but no layout of the threads covers them
+    (90, 1601, 9, 20, 12), (9, 1601, 100, 20, 2)]
 
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
