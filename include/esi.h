@@ -492,7 +492,8 @@ ESI_API long long esi_launch_count(const esi_ctx *ctx);
  */
 typedef struct esi_kernel_stat {
     char name[48];       /* e.g. "fd2_step[CGP|SMP]" */
-    long long launches;  /* kernel launches */
+    long long launches;  /* kernel launches; of a time loop its steps (a step may be two
+                            launches of half the shots, or part of one launch of many steps) */
     long long cells;     /* cell updates (or vector elements) processed */
     double bytes_per_cell;  /* algorithmic HBM bytes per cell update / element */
     double ms;           /* accumulated device time between the bracketing events */

@@ -168,12 +168,32 @@ struct esi_ctx {
     // the context stream; replays of an identical loop skip the per-step launch cost.
     struct GraphEntry {
         std::vector<unsigned char> key;
-        cudaGraphExec_t exec;
-        long long kernels;
-        unsigned long long used;
+        std::vector<cudaGraphExec_t> parts;   // launched in order
+        long long kernels = 0;
+        unsigned long long used = 0;
+        GraphEntry() = default;
+        GraphEntry(GraphEntry &&) = default;
+        GraphEntry &operator=(GraphEntry &&o) noexcept {
+            key.swap(o.key);
+            parts.swap(o.parts);
+            kernels = o.kernels;
+            used = o.used;
+            return *this;
+        }
+        ~GraphEntry() {
+            for (auto x : parts) cudaGraphExecDestroy(x);
+        }
     };
     std::vector<GraphEntry> graphs;
     cudaStream_t cap = nullptr;
+    // Concurrent chains of a time loop: the shots are independent systems, so a loop's steps run
+    // as one or two chains of launches, each over its own shots.  Chain 0 runs on the context
+    // stream (or the capture's), chain 1 on a stream forked from it and joined to it by events.
+    int chains = 1;
+    cudaStream_t chain_st = nullptr;
+    cudaEvent_t chain_ev[2] = {nullptr, nullptr};   // fork, join
+    int chain_shot(int c) const { return c * ns / chains; }   // its first shot (c = chains: the end)
+    cudaStream_t chain_stream(int c) const { return c ? chain_st : st; }
     bool use_graphs = true;
     bool pdl = true;               // loop steps after the first start as dependent launches
     unsigned long long graph_clock = 0;
@@ -201,8 +221,11 @@ struct esi_ctx {
     ~esi_ctx() {
         clear_groups();
         if (pc) pcnet_destroy(pc);
-        for (auto &g : graphs) cudaGraphExecDestroy(g.exec);
+        graphs.clear();
         if (cap) cudaStreamDestroy(cap);
+        if (chain_st) cudaStreamDestroy(chain_st);
+        for (auto e : chain_ev)
+            if (e) cudaEventDestroy(e);
         for (auto &p : pending) {
             cudaEventDestroy(p.a);
             cudaEventDestroy(p.b);
@@ -583,16 +606,71 @@ StepArgs<T> base_args(esi_ctx *ctx) {
 // One step of either kernel.  In 3D the step kernel samples its input state itself when
 // F_SMP is set (a.tout >= 0), by a gather of the receivers of each block's tile.
 template <typename T>
-esi_status step(esi_ctx *ctx, unsigned flags, const StepArgs<T> &a, bool chained = false) {
+esi_status step(esi_ctx *ctx, unsigned flags, const StepArgs<T> &a, bool chained = false,
+                int chain = -1) {
     StepArgs<T> b = a;
+    cudaStream_t st = ctx->st;
+    int ns = ctx->ns;
+    if (chain >= 0) {
+        st = ctx->chain_stream(chain);
+        b.s0 = ctx->chain_shot(chain);
+        ns = ctx->chain_shot(chain + 1) - b.s0;
+    }
     if (!state_map(ctx, a.cur, &b.tm) ||
         (ctx->g.ndim == 3 && (!state_map(ctx, a.po, &b.tm_old, 1) || !state_map(ctx, a.cc, &b.tm_cc, 2))))
         return ctx->fail(ESI_ERR_CUDA, "cuTensorMapEncodeTiled failed for a state buffer");
     if (ctx->g.ndim == 2) {
-        CKL(launch_step2<T>(flags, b, ctx->ns, ctx->st, chained && ctx->pdl));
+        CKL(launch_step2<T>(flags, b, ns, st, chained && ctx->pdl));
     } else {
         if (!(flags & F_SMP) || a.smp.nrec == 0) b.tout = -1;
-        CKL(launch_step3<T>(flags & ~F_SMP, b, ctx->ns, ctx->st, chained && ctx->pdl));
+        CKL(launch_step3<T>(flags & ~F_SMP, b, ns, st, chained && ctx->pdl));
+    }
+    return ESI_OK;
+}
+
+// Fork chain 1 from the context stream and join it again, whatever became of the launches
+// between (st).
+esi_status chains_fork(esi_ctx *ctx) {
+    if (ctx->chains == 1) return ESI_OK;
+    CK(cudaEventRecord(ctx->chain_ev[0], ctx->st));
+    CK(cudaStreamWaitEvent(ctx->chain_st, ctx->chain_ev[0], 0));
+    return ESI_OK;
+}
+esi_status chains_join(esi_ctx *ctx, esi_status st) {
+    if (ctx->chains == 1) return st;
+    cudaError_t e = cudaEventRecord(ctx->chain_ev[1], ctx->chain_st);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->st, ctx->chain_ev[1], 0);
+    if (e != cudaSuccess && st == ESI_OK)
+        st = ctx->fail(ESI_ERR_CUDA, std::string("joining the chains: ") + cudaGetErrorString(e));
+    return st;
+}
+
+// one step of every chain
+template <typename T>
+esi_status step_chains(esi_ctx *ctx, unsigned flags, const StepArgs<T> &a, bool chained) {
+    for (int c = 0; c < ctx->chains; ++c) {
+        esi_status st = step<T>(ctx, flags, a, chained, c);
+        if (st != ESI_OK) return st;
+    }
+    return ESI_OK;
+}
+
+// the DFT of a block of stashed states, or the block of sources of an inverse one, per chain
+template <typename T>
+esi_status dft_block_chains(esi_ctx *ctx, const T *snap, int K, int nf, const T *twid, T *acc) {
+    for (int c = 0; c < ctx->chains; ++c) {
+        const int s0 = ctx->chain_shot(c);
+        CKL(launch_dft_block<T>(snap, K, ctx->ns, s0, ctx->chain_shot(c + 1) - s0, ctx->sst, ctx->g.nx,
+                                ctx->px, nf, twid, acc, ctx->chain_stream(c)));
+    }
+    return ESI_OK;
+}
+template <typename T>
+esi_status idft_block_chains(esi_ctx *ctx, const T *qb, int K, int kst, int nf, const T *tw, T *src) {
+    for (int c = 0; c < ctx->chains; ++c) {
+        const int s0 = ctx->chain_shot(c);
+        CKL(launch_idft_block<T>(qb, K, kst, ctx->ns, s0, ctx->chain_shot(c + 1) - s0, ctx->sst, nf, tw,
+                                 src, ctx->chain_stream(c)));
     }
     return ESI_OK;
 }
@@ -836,6 +914,30 @@ struct LoopSmpHost {
     }
 };
 
+// How many chains the time loops run in: two for 2D FP32 steps of more blocks than the chip
+// holds at once.  A step ends in a latency of about 3 us (the last wave's loads, its stores, the
+// next step's first tile) and in a partly filled last wave; the other chain's blocks fill both.
+// Measured, 1000 steps of a forward loop in one and in two chains, ms: 624 blocks (6 shots of
+// 801 x 241) 5.21 -> 4.24, 1664 blocks (16 of them) 9.82 -> 7.72, 12160 blocks (64 shots of
+// 1201 x 301) 71.0 -> 67.3; three and four chains give no more (9.72 and 9.79 -> 7.73 for the
+// 1664).  Up to one wave (608 blocks) there is nothing to fill: 448 blocks 4.18 either way, and
+// the second launch is lost.  FP64 steps are bound by the FP64 units and the 3D steps by their
+// marching chains: equal in one and in two.
+template <typename T>
+esi_status setup_chains(esi_ctx *ctx) {
+    ctx->chains = 1;
+    if (sizeof(T) != 4 || ctx->g.ndim != 2 || ctx->ns < 2 || ctx->lp.ok) return ESI_OK;
+    int dev = 0, nsm = 0;
+    CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    if ((long long)ctx->ntiles * ctx->ns <= (long long)nsm * MINB2) return ESI_OK;
+    if (!ctx->chain_st) CK(cudaStreamCreateWithFlags(&ctx->chain_st, cudaStreamNonBlocking));
+    for (auto &ev : ctx->chain_ev)
+        if (!ev) CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+    ctx->chains = 2;
+    return ESI_OK;
+}
+
 // Chooses the cut of the on-chip loops: the cheapest whose tiles, with their point lists, fit in
 // shared memory and whose shots fit on the SMs; none (per-step kernel) when not even one shot
 // fits on the chip.
@@ -938,6 +1040,7 @@ esi_status setup_geometry(esi_ctx *ctx) {
     if ((e = build_smp<T>(ctx, ctx->smp_rec, rec_smp)) != ESI_OK) return e;
     if ((e = build_smp<T>(ctx, ctx->smp_src, src_smp)) != ESI_OK) return e;
     if ((e = setup_loops<T>(ctx, src_inj, rec_inj, rec_smp, src_smp)) != ESI_OK) return e;
+    if ((e = setup_chains<T>(ctx)) != ESI_OK) return e;
     CK(upload(ctx->src_pos, ctx->src_xyz, ctx->st));
     return ESI_OK;
 }
@@ -967,6 +1070,7 @@ esi_status check_dev_err(esi_ctx *ctx) {
 
 // ------------------------------------------------------------------ loop graphs
 constexpr int GRAPH_MIN_STEPS = 32;   // shorter loops are launched directly
+constexpr int GRAPH_PART = 256;        // steps captured at a time
 constexpr size_t GRAPH_CACHE = 8;      // instantiated loops kept per context
 
 template <typename T>
@@ -991,11 +1095,13 @@ std::vector<unsigned char> loop_key(const StepArgs<T> &a, unsigned flags, int di
 bool graph_replay(esi_ctx *ctx, const std::vector<unsigned char> &key, esi_status &st) {
     for (auto &g : ctx->graphs)
         if (g.key == key) {
-            cudaError_t e = cudaGraphLaunch(g.exec, ctx->st);
-            if (e != cudaSuccess) {
-                st = ctx->fail(ESI_ERR_CUDA, std::string("cudaGraphLaunch: ") + cudaGetErrorString(e));
-            } else {
-                st = ESI_OK;
+            st = ESI_OK;
+            for (size_t i = 0; i < g.parts.size() && st == ESI_OK; ++i) {
+                cudaError_t e = cudaGraphLaunch(g.parts[i], ctx->st);
+                if (e != cudaSuccess)
+                    st = ctx->fail(ESI_ERR_CUDA, std::string("cudaGraphLaunch: ") + cudaGetErrorString(e));
+            }
+            if (st == ESI_OK) {
                 ctx->launches += g.kernels;
                 g.used = ++ctx->graph_clock;
             }
@@ -1004,43 +1110,56 @@ bool graph_replay(esi_ctx *ctx, const std::vector<unsigned char> &key, esi_statu
     return false;
 }
 
-// Capture `body` (which enqueues on ctx->st) into a graph, cache it and launch it.
+// Run a loop of `steps` steps, body(i0, i1) enqueueing the steps [i0, i1) on ctx->st: replayed
+// when it is cached, else captured and cached.  The capture goes in parts of at least
+// GRAPH_PART steps (a multiple of `unit`), each launched as soon as it is instantiated, so that
+// the GPU runs one part while the host captures the next (about 3 us a launch).  Measured, 1000
+// steps of 4 shots of 801 x 241 on new buffers: 6.7 ms captured whole, 4.8 / 4.6 / 4.4 in parts
+// of 256 / 128 / 64; replayed 4.17, 4.17 / 4.18 / 4.22 (a boundary costs the overlap of two steps).
 template <typename F>
-esi_status graph_capture(esi_ctx *ctx, std::vector<unsigned char> &&key, F &&body) {
+esi_status graph_run(esi_ctx *ctx, std::vector<unsigned char> &&key, int steps, int unit, F &&body) {
+    esi_status st = ESI_OK;
+    if (graph_replay(ctx, key, st)) return st;
     if (!ctx->cap) CK(cudaStreamCreateWithFlags(&ctx->cap, cudaStreamNonBlocking));
+    const int len = (GRAPH_PART + unit - 1) / unit * unit;
+    esi_ctx::GraphEntry entry;
+    entry.key = std::move(key);
+    entry.parts.reserve(steps / len + 1);
     std::lock_guard<std::recursive_mutex> lk(g_dev_mu);   // no allocation meets the capture
     cudaStream_t user = ctx->st;
     const long long l0 = ctx->launches;
-    CK(cudaStreamBeginCapture(ctx->cap, cudaStreamCaptureModeThreadLocal));
-    ctx->st = ctx->cap;
-    esi_status e = body();
-    ctx->st = user;
-    cudaGraph_t graph = nullptr;
-    cudaError_t ce = cudaStreamEndCapture(ctx->cap, &graph);
-    if (e != ESI_OK) {
-        if (graph) cudaGraphDestroy(graph);
-        return e;
+    for (int i0 = 0; i0 < steps; i0 += len) {
+        CK(cudaStreamBeginCapture(ctx->cap, cudaStreamCaptureModeThreadLocal));
+        ctx->st = ctx->cap;
+        st = body(i0, std::min(steps, i0 + len));
+        ctx->st = user;
+        cudaGraph_t graph = nullptr;
+        cudaError_t ce = cudaStreamEndCapture(ctx->cap, &graph);
+        if (st != ESI_OK) {
+            if (graph) cudaGraphDestroy(graph);
+            return st;
+        }
+        if (ce != cudaSuccess) return ctx->fail(ESI_ERR_CUDA, std::string("capture: ") + cudaGetErrorString(ce));
+        cudaGraphExec_t exec = nullptr;
+        ce = cudaGraphInstantiate(&exec, graph, 0);
+        cudaGraphDestroy(graph);
+        if (ce != cudaSuccess)
+            return ctx->fail(ESI_ERR_CUDA, std::string("cudaGraphInstantiate: ") + cudaGetErrorString(ce));
+        entry.parts.push_back(exec);
+        ce = cudaGraphLaunch(exec, ctx->st);
+        if (ce != cudaSuccess)
+            return ctx->fail(ESI_ERR_CUDA, std::string("cudaGraphLaunch: ") + cudaGetErrorString(ce));
     }
-    if (ce != cudaSuccess) return ctx->fail(ESI_ERR_CUDA, std::string("capture: ") + cudaGetErrorString(ce));
-    cudaGraphExec_t exec = nullptr;
-    ce = cudaGraphInstantiate(&exec, graph, 0);
-    cudaGraphDestroy(graph);
-    if (ce != cudaSuccess)
-        return ctx->fail(ESI_ERR_CUDA, std::string("cudaGraphInstantiate: ") + cudaGetErrorString(ce));
-    const long long kernels = ctx->launches - l0;
-    ctx->launches = l0;  // counted when the graph runs
-    if (ctx->graphs.size() >= GRAPH_CACHE) {
-        auto lru = std::min_element(ctx->graphs.begin(), ctx->graphs.end(),
-                                    [](const esi_ctx::GraphEntry &x, const esi_ctx::GraphEntry &y) {
-                                        return x.used < y.used;
-                                    });
-        cudaGraphExecDestroy(lru->exec);
-        ctx->graphs.erase(lru);
-    }
-    ctx->graphs.push_back({std::move(key), exec, kernels, ++ctx->graph_clock});
-    esi_status st;
-    graph_replay(ctx, ctx->graphs.back().key, st);
-    return st;
+    entry.kernels = ctx->launches - l0;
+    entry.used = ++ctx->graph_clock;
+    if (ctx->graphs.size() >= GRAPH_CACHE)
+        *std::min_element(ctx->graphs.begin(), ctx->graphs.end(),
+                          [](const esi_ctx::GraphEntry &x, const esi_ctx::GraphEntry &y) {
+                              return x.used < y.used;
+                          }) = std::move(entry);
+    else
+        ctx->graphs.push_back(std::move(entry));
+    return ESI_OK;
 }
 
 // ------------------------------------------------------------------ on-chip loops (2D)
@@ -1101,20 +1220,20 @@ esi_status fwd_loop(esi_ctx *ctx, StepArgs<T> a, unsigned flags, T *&cur, T *&po
     (void)ckpt_at;
     cudaEvent_t ev = prof_mark(ctx);
     T *c0 = cur, *p0 = po;
-    auto body = [&]() -> esi_status {
-        T *c = c0, *q = p0;
-        for (int n = n0; n < n1; ++n) {
+    auto body = [&](int i0, int i1) -> esi_status {
+        T *c = i0 & 1 ? p0 : c0, *q = i0 & 1 ? c0 : p0;
+        esi_status e = chains_fork(ctx);
+        for (int n = n0 + i0; n < n0 + i1 && e == ESI_OK; ++n) {
             a.cur = c;
             a.po = q;
             a.n = n;
             a.tin = n;
             a.tout = n - 1;
             a.slot_w = n - n0;
-            esi_status e = step<T>(ctx, flags, a, n > n0);
-            if (e != ESI_OK) return e;
+            e = step_chains<T>(ctx, flags, a, n > n0 + i0);
             std::swap(c, q);
         }
-        return ESI_OK;
+        return chains_join(ctx, e);
     };
     esi_status e;
     if (loop_ready(ctx, n1 - n0)) {
@@ -1124,9 +1243,9 @@ esi_status fwd_loop(esi_ctx *ctx, StepArgs<T> a, unsigned flags, T *&cur, T *&po
         e = loop_run<T>(ctx, flags, a, c0, p0, n1 - n0, +1);
     } else if (ctx->use_graphs && n1 - n0 >= GRAPH_MIN_STEPS) {
         auto key = loop_key(a, flags, +1, n0, n1, false, c0, p0);
-        if (!graph_replay(ctx, key, e)) e = graph_capture(ctx, std::move(key), body);
+        e = graph_run(ctx, std::move(key), n1 - n0, 1, body);
     } else {
-        e = body();
+        e = body(0, n1 - n0);
     }
     if (e != ESI_OK) return e;
     if ((n1 - n0) & 1) std::swap(cur, po);
@@ -1142,40 +1261,40 @@ template <typename T>
 esi_status fwd_dft_loop(esi_ctx *ctx, StepArgs<T> a, unsigned flags, T *cur, T *po, T *tr) {
     cudaEvent_t ev = prof_mark(ctx);
     const int nt = ctx->nt;
-    auto body = [&]() -> esi_status {
-        T *c = cur, *q = po;
-        for (int n0 = 0; n0 < nt; n0 += ctx->dft_k) {
-            const int n1 = std::min(nt, n0 + ctx->dft_k);
+    auto body = [&](int i0, int i1) -> esi_status {
+        T *c = i0 & 1 ? po : cur, *q = i0 & 1 ? cur : po;
+        esi_status e = chains_fork(ctx);
+        for (int n0 = i0; n0 < i1 && e == ESI_OK; n0 += ctx->dft_k) {
+            const int n1 = std::min(i1, n0 + ctx->dft_k);
             if (loop_ready(ctx, n1 - n0)) {
                 a.n = a.tin = n0;
                 a.tout = n0 - 1;
                 a.slot_w = 0;
-                esi_status e = loop_run<T>(ctx, flags, a, c, q, n1 - n0, +1);
-                if (e != ESI_OK) return e;
+                e = loop_run<T>(ctx, flags, a, c, q, n1 - n0, +1);
                 if ((n1 - n0) & 1) std::swap(c, q);
-            } else for (int n = n0; n < n1; ++n) {
+            } else for (int n = n0; n < n1 && e == ESI_OK; ++n) {
                 a.cur = c;
                 a.po = q;
                 a.n = n;
                 a.tin = n;
                 a.tout = n - 1;
                 a.slot_w = n - n0;
-                esi_status e = step<T>(ctx, flags, a, n > 0);
-                if (e != ESI_OK) return e;
+                e = step_chains<T>(ctx, flags, a, n > i0);
                 std::swap(c, q);
             }
-            CKL(launch_dft_block<T>(a.stash_w, n1 - n0, ctx->ns, ctx->sst, ctx->g.nx, ctx->px, a.nf,
-                                    a.twid + (size_t)n0 * a.nf * 2, a.dft, ctx->st));
+            if (e == ESI_OK)
+                e = dft_block_chains<T>(ctx, a.stash_w, n1 - n0, a.nf, a.twid + (size_t)n0 * a.nf * 2, a.dft);
         }
-        CKL(launch_sample_global<T>(a.smp, c, ctx->sst, tr, nt - 1, ctx->st));
+        if ((e = chains_join(ctx, e)) != ESI_OK) return e;
+        if (i1 == nt) CKL(launch_sample_global<T>(a.smp, c, ctx->sst, tr, nt - 1, ctx->st));
         return ESI_OK;
     };
     esi_status e;
     if (ctx->use_graphs && nt >= GRAPH_MIN_STEPS && !loop_ready(ctx, ctx->dft_k)) {
         auto key = loop_key(a, flags, +2, 0, nt, false, cur, po);
-        if (!graph_replay(ctx, key, e)) e = graph_capture(ctx, std::move(key), body);
+        e = graph_run(ctx, std::move(key), nt, ctx->dft_k, body);
     } else {
-        e = body();
+        e = body(0, nt);
     }
     if (e != ESI_OK) return e;
     // the stencil and the stash store per step, plus the block pass: the stash once more
@@ -1326,9 +1445,10 @@ esi_status adj_loop(esi_ctx *ctx, StepArgs<T> a, unsigned flags, T *&cur, T *&po
                     int j0, bool sample_src) {
     cudaEvent_t ev = prof_mark(ctx);
     T *c0 = cur, *p0 = po;
-    auto body = [&]() -> esi_status {
-        T *c = c0, *q = p0;
-        for (int j = j1; j > j0; --j) {
+    auto body = [&](int i0, int i1) -> esi_status {
+        T *c = i0 & 1 ? p0 : c0, *q = i0 & 1 ? c0 : p0;
+        esi_status e = chains_fork(ctx);
+        for (int j = j1 - i0; j > j1 - i1 && e == ESI_OK; --j) {
             a.cur = c;
             a.po = q;
             a.n = j - 1;
@@ -1336,11 +1456,10 @@ esi_status adj_loop(esi_ctx *ctx, StepArgs<T> a, unsigned flags, T *&cur, T *&po
             a.nout = j - 1;
             a.tout = (sample_src && j <= ctx->nt - 1) ? j : -1;
             a.slot_r = (j - 1) - j0;
-            esi_status e = step<T>(ctx, flags, a, j < j1);
-            if (e != ESI_OK) return e;
+            e = step_chains<T>(ctx, flags, a, j < j1 - i0);
             std::swap(c, q);
         }
-        return ESI_OK;
+        return chains_join(ctx, e);
     };
     esi_status e;
     if (loop_ready(ctx, j1 - j0)) {
@@ -1350,9 +1469,9 @@ esi_status adj_loop(esi_ctx *ctx, StepArgs<T> a, unsigned flags, T *&cur, T *&po
         e = loop_run<T>(ctx, flags, a, c0, p0, j1 - j0, -1);
     } else if (ctx->use_graphs && j1 - j0 >= GRAPH_MIN_STEPS) {
         auto key = loop_key(a, flags, -1, j0, j1, sample_src, c0, p0);
-        if (!graph_replay(ctx, key, e)) e = graph_capture(ctx, std::move(key), body);
+        e = graph_run(ctx, std::move(key), j1 - j0, 1, body);
     } else {
-        e = body();
+        e = body(0, j1 - j0);
     }
     if (e != ESI_OK) return e;
     if ((j1 - j0) & 1) std::swap(cur, po);
@@ -2246,18 +2365,18 @@ esi_status fdcg_impl(esi_ctx *ctx, double lambda, double tol, int max_iter, cons
         a.twid = fold_d + (size_t)part * nt * nf * 2;
         a.dft = out;
         T *c0 = ctx->a0.as<T>(), *p0 = ctx->a1.as<T>();
-        auto body = [&]() -> esi_status {
-            T *c = c0, *q = p0;
-            for (int jhi = nt; jhi > 0;) {
-                const int jlo = std::max(0, jhi - K);
+        auto body = [&](int i0, int i1) -> esi_status {
+            T *c = i0 & 1 ? p0 : c0, *q = i0 & 1 ? c0 : p0;
+            esi_status st = chains_fork(ctx);
+            for (int jhi = nt - i0; jhi > nt - i1 && st == ESI_OK;) {
+                const int jlo = std::max(nt - i1, jhi - K);
                 if (loop_ready(ctx, jhi - jlo)) {
                     a.n = a.tin = a.nout = jhi - 1;
                     a.tout = -1;
                     a.slot_w = jhi - 1 - jlo;
-                    esi_status st = loop_run<T>(ctx, aflags, a, c, q, jhi - jlo, -1);
-                    if (st != ESI_OK) return st;
+                    st = loop_run<T>(ctx, aflags, a, c, q, jhi - jlo, -1);
                     if ((jhi - jlo) & 1) std::swap(c, q);
-                } else for (int j = jhi; j > jlo; --j) {
+                } else for (int j = jhi; j > jlo && st == ESI_OK; --j) {
                     a.cur = c;
                     a.po = q;
                     a.n = j - 1;
@@ -2265,22 +2384,21 @@ esi_status fdcg_impl(esi_ctx *ctx, double lambda, double tol, int max_iter, cons
                     a.nout = j - 1;
                     a.tout = -1;
                     a.slot_w = (j - 1) - jlo;   // slots in time order within the block
-                    esi_status st = step<T>(ctx, aflags, a, j < nt);
-                    if (st != ESI_OK) return st;
+                    st = step_chains<T>(ctx, aflags, a, j < nt - i0);
                     std::swap(c, q);
                 }
-                CKL(launch_dft_block<T>(a.stash_w, jhi - jlo, ns, ctx->sst, ctx->g.nx, ctx->px, nf,
-                                        a.twid + (size_t)jlo * nf * 2, out, ctx->st));
+                if (st == ESI_OK)
+                    st = dft_block_chains<T>(ctx, a.stash_w, jhi - jlo, nf, a.twid + (size_t)jlo * nf * 2, out);
                 jhi = jlo;
             }
-            return ESI_OK;
+            return chains_join(ctx, st);
         };
         esi_status st;
         if (ctx->use_graphs && nt >= GRAPH_MIN_STEPS && !loop_ready(ctx, K)) {
             auto key = loop_key(a, aflags, -3, part, nt, false, c0, p0);
-            if (!graph_replay(ctx, key, st)) st = graph_capture(ctx, std::move(key), body);
+            st = graph_run(ctx, std::move(key), nt, K, body);
         } else {
-            st = body();
+            st = body(0, nt);
         }
         if (st != ESI_OK) return st;
         prof_close(ctx, ev, step_name(ctx, aflags) + "+dft_block",
@@ -2305,39 +2423,39 @@ esi_status fdcg_impl(esi_ctx *ctx, double lambda, double tol, int max_iter, cons
         a.nf = nf;
         a.twid = syn_d + (size_t)part * nt * nf * 2;
         T *c0 = ctx->u0.as<T>(), *p0 = ctx->u1.as<T>();
-        auto body = [&]() -> esi_status {
-            T *c = c0, *q = p0;
-            for (int n0 = 0; n0 < nt; n0 += K) {
-                const int n1 = std::min(nt, n0 + K);
-                CKL(launch_idft_block<T>(qb, n1 - n0, K, ns, ctx->sst, nf,
-                                         a.twid + (size_t)n0 * nf * 2, src, ctx->st));
+        auto body = [&](int i0, int i1) -> esi_status {
+            T *c = i0 & 1 ? p0 : c0, *q = i0 & 1 ? c0 : p0;
+            esi_status st = chains_fork(ctx);
+            for (int n0 = i0; n0 < i1 && st == ESI_OK; n0 += K) {
+                const int n1 = std::min(i1, n0 + K);
+                st = idft_block_chains<T>(ctx, qb, n1 - n0, K, nf, a.twid + (size_t)n0 * nf * 2, src);
+                if (st != ESI_OK) break;
                 if (loop_ready(ctx, n1 - n0)) {
                     a.n = 0;   // the stash slot
                     a.tin = n0;
                     a.tout = n0 - 1;
-                    esi_status st = loop_run<T>(ctx, F_CGP | F_SMP, a, c, q, n1 - n0, +1);
-                    if (st != ESI_OK) return st;
+                    st = loop_run<T>(ctx, F_CGP | F_SMP, a, c, q, n1 - n0, +1);
                     if ((n1 - n0) & 1) std::swap(c, q);
-                } else for (int n = n0; n < n1; ++n) {
+                } else for (int n = n0; n < n1 && st == ESI_OK; ++n) {
                     a.cur = c;
                     a.po = q;
                     a.n = n - n0;   // the stash slot
                     a.tin = n;
                     a.tout = n - 1;
-                    esi_status st = step<T>(ctx, F_CGP | F_SMP, a, n > 0);
-                    if (st != ESI_OK) return st;
+                    st = step_chains<T>(ctx, F_CGP | F_SMP, a, n > i0);
                     std::swap(c, q);
                 }
             }
-            CKL(launch_sample_global<T>(a.smp, c, ctx->sst, tr, nt - 1, ctx->st));
+            if ((st = chains_join(ctx, st)) != ESI_OK) return st;
+            if (i1 == nt) CKL(launch_sample_global<T>(a.smp, c, ctx->sst, tr, nt - 1, ctx->st));
             return ESI_OK;
         };
         esi_status st;
         if (ctx->use_graphs && nt >= GRAPH_MIN_STEPS && !loop_ready(ctx, K)) {
             auto key = loop_key(a, F_CGP | F_SMP, +3, part, nt, false, c0, p0);
-            if (!graph_replay(ctx, key, st)) st = graph_capture(ctx, std::move(key), body);
+            st = graph_run(ctx, std::move(key), nt, K, body);
         } else {
-            st = body();
+            st = body(0, nt);
         }
         if (st != ESI_OK) return st;
         prof_close(ctx, ev, step_name(ctx, F_CGP | F_SMP) + "+idft_block",

@@ -35,6 +35,7 @@ constexpr int TX2 = 64;             // tile width (x) of the 2D step kernel
 #endif
 constexpr int TZ2 = ESI_TZ2;        // tile height (z)
 constexpr int NT2 = 256;            // threads per block of the 2D step kernel
+constexpr int MINB2 = 4;            // its resident blocks per SM, which the registers must allow
 constexpr int SW2 = TX2 + 2 * HALO; // shared tile width incl. halo (72: 16-byte rows)
 constexpr int SH2 = TZ2 + 2 * HALO; // shared tile height incl. halo
 constexpr int MAXP = 8;             // interpolation points per receiver (4 in 2D, 8 in 3D)
@@ -111,6 +112,7 @@ struct StepArgs {
     int opx;                   // row pitch of the F_OUT target (nx: caller, px: internal)
     long long oplane, ofst;    // its plane and shot strides
     int ntx, nty, ntz;         // tiles per shot
+    int s0;                    // first shot of a 2D launch
     const T *cur;              // input state
     T *po;                     // in: older state, out: new state
     const T *cc;               // [nz][ny][px] v^2 dt^2 / dx^2
@@ -338,21 +340,22 @@ constexpr int DFT_BLOCK_MAX = 64;
 int dft_block_steps(long long stash_plane_bytes, size_t device_bytes);
 
 // Blocked DTFT: acc [ns][nf][sst][2] += sum_k snap[k][ns][sst] (cos, sin)(twid[k][nf]) over the
-// K <= DFT_BLOCK_MAX stashed states of one block.  Rows of px cells of which nx are real:
-// 16-byte chunks that lie wholly in the pad are skipped (the step kernels never write them,
-// so the stash holds whatever the memory held there; the accumulators keep their zero pads).
+// K <= DFT_BLOCK_MAX stashed states of one block, for the shots [s0, s0 + nsl).  Rows of px
+// cells of which nx are real: 16-byte chunks that lie wholly in the pad are skipped (the step
+// kernels never write them, so the stash holds whatever the memory held there; the accumulators
+// keep their zero pads).
 template <typename T>
-cudaError_t launch_dft_block(const T *snap, int K, int ns, long long sst, int nx, int px, int nf,
-                             const T *twid, T *acc, cudaStream_t st);
+cudaError_t launch_dft_block(const T *snap, int K, int ns, int s0, int nsl, long long sst, int nx,
+                             int px, int nf, const T *twid, T *acc, cudaStream_t st);
 
 // Frequency-domain ESI (Eq. "idtft", "normaldtft"), at most FD_MAXF frequencies.
 constexpr int FD_MAXF = 8;
 // inverse DTFT of one block: src[s][k][cell] = sum_m re(qb_m) tw[k][m].x + im(qb_m) tw[k][m].y
-// for the K <= kst steps of the block (kst slots per shot), qb pitched complex slices
-// [ns][nf][sst][2]
+// for the K <= kst steps of the block (kst slots per shot) and the shots [s0, s0 + nsl),
+// qb pitched complex slices [ns][nf][sst][2]
 template <typename T>
-cudaError_t launch_idft_block(const T *qb, int K, int kst, int ns, long long sst, int nf,
-                              const T *tw, T *src, cudaStream_t st);
+cudaError_t launch_idft_block(const T *qb, int K, int kst, int ns, int s0, int nsl, long long sst,
+                              int nf, const T *tw, T *src, cudaStream_t st);
 // out_m += pb2 * sum_m' G[m][m'] p_m' per cell (G = F F^H / nt, complex [nf][nf][2]) and the
 // per-block partials of Re <p, out> ([ns][DVEC_NBLK]); inactive shots skipped
 template <typename T>

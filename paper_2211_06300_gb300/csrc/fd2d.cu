@@ -21,11 +21,6 @@
 //              on-the-fly DTFT accumulation.
 #include "esi_internal.h"
 
-// resident blocks per SM the register allocation must allow (256 threads each)
-#ifndef ESI_FD2_MINB
-#define ESI_FD2_MINB 4
-#endif
-
 namespace esi {
 namespace {
 
@@ -80,7 +75,7 @@ __device__ __forceinline__ void stv(T *p, const Vec<T> &v) {
 }
 
 template <typename T, unsigned F>
-__global__ void __launch_bounds__(NT2, ESI_FD2_MINB) fd2_step_kernel(const __grid_constant__ StepArgs<T> a) {
+__global__ void __launch_bounds__(NT2, MINB2) fd2_step_kernel(const __grid_constant__ StepArgs<T> a) {
     constexpr int VEC = Vec<T>::n;     // cells per thread-vector
     constexpr int TPR = TX2 / VEC;     // threads per tile row
     constexpr int RPP = NT2 / TPR;     // rows per pass
@@ -90,7 +85,7 @@ __global__ void __launch_bounds__(NT2, ESI_FD2_MINB) fd2_step_kernel(const __gri
     __shared__ __align__(8) unsigned long long bar;
     __shared__ __align__(16) T qpt[(F & F_PT) ? TZ2 * TX2 : VEC];
     const int tid = threadIdx.x;
-    const int s = blockIdx.z;
+    const int s = a.s0 + blockIdx.z;
     if (a.active && !a.active[s]) return;
     const int x0 = blockIdx.x * TX2, z0 = blockIdx.y * TZ2;
     const int tile = (s * a.ntz + blockIdx.y) * a.ntx + blockIdx.x;

@@ -1010,8 +1010,8 @@ cudaError_t launch_fd_precond(T *z, const T *r, const T *w, int nf, int ns, long
 }
 
 template <typename T>
-cudaError_t launch_idft_block(const T *qb, int K, int kst, int ns, long long sst, int nf,
-                              const T *tw, T *src, cudaStream_t st) {
+cudaError_t launch_idft_block(const T *qb, int K, int kst, int ns, int s0, int nsl, long long sst,
+                              int nf, const T *tw, T *src, cudaStream_t st) {
     if (nf < 1 || nf > FD_MAXF || K < 1 || K > kst || K > DFT_BLOCK_MAX) return cudaErrorInvalidValue;
     // the resident blocks, shared among the shots (grid-stride over the cells)
     static PerDevice slots;
@@ -1030,8 +1030,8 @@ cudaError_t launch_idft_block(const T *qb, int K, int kst, int ns, long long sst
         }) != cudaSuccess)
         nres = 1024;
     const int per_shot = std::max(1, nres / std::max(1, ns));
-    idft_block_kernel<T><<<dim3(blocks_for(sst / V16<T>::n, per_shot), ns), RT, 0, st>>>(
-        qb, K, kst, ns, sst, nf, tw, src);
+    idft_block_kernel<T><<<dim3(blocks_for(sst / V16<T>::n, per_shot), nsl), RT, 0, st>>>(
+        qb + (long long)s0 * nf * sst * 2, K, kst, ns, sst, nf, tw, src + (long long)s0 * kst * sst);
     return cudaGetLastError();
 }
 
@@ -1065,12 +1065,12 @@ int dft_block_slots() {
 }
 
 template <typename T, int M>
-cudaError_t go_dft_block(const T *snap, int K, int ns, long long sst, int nx, int px, int nf,
-                         const T *twid, T *acc, cudaStream_t st) {
+cudaError_t go_dft_block(const T *snap, int K, int ns, int s0, int nsl, long long sst, int nx, int px,
+                         int nf, const T *twid, T *acc, cudaStream_t st) {
     // the resident blocks, shared among the shots
     const int per_shot = std::max(1, dft_block_slots<T, M>() / std::max(1, ns));
-    dft_block_kernel<T, M><<<dim3(blocks_for(sst / V16<T>::n, per_shot), ns), RT, 0, st>>>(
-        snap, K, ns, sst, nx, px, nf, twid, acc);
+    dft_block_kernel<T, M><<<dim3(blocks_for(sst / V16<T>::n, per_shot), nsl), RT, 0, st>>>(
+        snap + s0 * sst, K, ns, sst, nx, px, nf, twid, acc + (long long)s0 * nf * sst * 2);
     return cudaGetLastError();
 }
 }  // namespace
@@ -1085,18 +1085,18 @@ int dft_block_steps(long long stash_plane_bytes, size_t device_bytes) {
 }
 
 template <typename T>
-cudaError_t launch_dft_block(const T *snap, int K, int ns, long long sst, int nx, int px, int nf,
-                             const T *twid, T *acc, cudaStream_t st) {
+cudaError_t launch_dft_block(const T *snap, int K, int ns, int s0, int nsl, long long sst, int nx,
+                             int px, int nf, const T *twid, T *acc, cudaStream_t st) {
     if (K < 1 || K > DFT_BLOCK_MAX || nf < 1) return cudaErrorInvalidValue;
     switch (std::min(nf, DFT_MCH)) {
-        case 1: return go_dft_block<T, 1>(snap, K, ns, sst, nx, px, nf, twid, acc, st);
-        case 2: return go_dft_block<T, 2>(snap, K, ns, sst, nx, px, nf, twid, acc, st);
-        case 3: return go_dft_block<T, 3>(snap, K, ns, sst, nx, px, nf, twid, acc, st);
-        case 4: return go_dft_block<T, 4>(snap, K, ns, sst, nx, px, nf, twid, acc, st);
-        case 5: return go_dft_block<T, 5>(snap, K, ns, sst, nx, px, nf, twid, acc, st);
-        case 6: return go_dft_block<T, 6>(snap, K, ns, sst, nx, px, nf, twid, acc, st);
-        case 7: return go_dft_block<T, 7>(snap, K, ns, sst, nx, px, nf, twid, acc, st);
-        default: return go_dft_block<T, 8>(snap, K, ns, sst, nx, px, nf, twid, acc, st);
+        case 1: return go_dft_block<T, 1>(snap, K, ns, s0, nsl, sst, nx, px, nf, twid, acc, st);
+        case 2: return go_dft_block<T, 2>(snap, K, ns, s0, nsl, sst, nx, px, nf, twid, acc, st);
+        case 3: return go_dft_block<T, 3>(snap, K, ns, s0, nsl, sst, nx, px, nf, twid, acc, st);
+        case 4: return go_dft_block<T, 4>(snap, K, ns, s0, nsl, sst, nx, px, nf, twid, acc, st);
+        case 5: return go_dft_block<T, 5>(snap, K, ns, s0, nsl, sst, nx, px, nf, twid, acc, st);
+        case 6: return go_dft_block<T, 6>(snap, K, ns, s0, nsl, sst, nx, px, nf, twid, acc, st);
+        case 7: return go_dft_block<T, 7>(snap, K, ns, s0, nsl, sst, nx, px, nf, twid, acc, st);
+        default: return go_dft_block<T, 8>(snap, K, ns, s0, nsl, sst, nx, px, nf, twid, acc, st);
     }
 }
 
@@ -1277,11 +1277,11 @@ cudaError_t launch_mlincomb(T *z, double alpha, const T *x, double beta, const T
                                             double, double, cudaStream_t);                       \
     template cudaError_t launch_fd_precond<T>(T *, const T *, const T *, int, int, long long,     \
                                               const int *, double *, cudaStream_t);              \
-    template cudaError_t launch_idft_block<T>(const T *, int, int, int, long long, int, const T *, \
-                                              T *, cudaStream_t);                                \
+    template cudaError_t launch_idft_block<T>(const T *, int, int, int, int, int, long long, int,   \
+                                              const T *, T *, cudaStream_t);                     \
     template cudaError_t launch_fd_b2g_dot<T>(T *, const T *, const T *, const double *, int, int, \
                                               long long, const int *, double *, cudaStream_t);   \
-    template cudaError_t launch_dft_block<T>(const T *, int, int, long long, int, int, int,      \
+    template cudaError_t launch_dft_block<T>(const T *, int, int, int, int, long long, int, int, int, \
                                              const T *, T *, cudaStream_t);
 
 ESI_INST(float)
