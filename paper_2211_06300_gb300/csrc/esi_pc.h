@@ -38,12 +38,13 @@ constexpr long long param_count() {
     return n;
 }
 
-// activation map [n][H][W][C_] BF16, box (8 channels, 130 columns, 1 row, 1 image)
+// activation map [n][H][W][C_] BF16, box (one row of 130 pixels), swizzled
 cudaError_t make_act_map(CUtensorMap *tm, const void *base, int C_, int W, int H, int n);
 // conv epilogue options
 struct ConvEpi {
     const float *oscale = nullptr;   // per-image output factor (applied after the activation)
     const float *irms = nullptr;     // per-image input RMS: the accumulator is divided by it
+    int wide = 0;                    // (set by the launch) the output is 32-byte aligned
     int nchw = 0;                    // output planes [img][c][H][W] instead of channels-last
 };
 template <int CIN, int COUT, bool RELU, typename OUT>

@@ -10,10 +10,9 @@
 // Activations are BF16, channels-last [img][h][w][c].  Every 3 x 3 convolution is an
 // implicit GEMM on the 5th-generation tensor cores: a tile is 128 output pixels of one row
 // (M = 128), N = output channels, and each of the 9 taps contributes K = input channels.
-// The 3-row input patch of a tile is staged by TMA (one box per 8-channel chunk, zero fill
-// at the image edges) in the canonical no-swizzle K-major layout, so every tap is the same
-// patch seen through a shared-memory descriptor shifted by (dy * 130 + dx) * 16 bytes.  One
-// thread issues tcgen05.mma into a TMEM accumulator; the four warps read it back with
+// The input rows of a tile are staged by TMA (one box of whole pixels per row, zero fill at the
+// image edges) in a swizzled K-major layout, so every tap is one of three rows seen through a
+// shared-memory descriptor shifted by dx pixels.  One thread issues tcgen05.mma into a TMEM accumulator; the four warps read it back with
 // tcgen05.ld for the bias / ReLU / BF16 epilogue.  Training reuses the same kernel for the
 // input gradient (flipped, transposed weights); the weight gradient, whose M is only 16 or
 // 32 channels (below the tcgen05 minimum of 64 rows), runs on warp-level mma.sync.
@@ -30,19 +29,22 @@ namespace {
 
 constexpr int TM = 128;              // output pixels per conv tile
 constexpr int PW = TM + 2;           // patch width (1-pixel halo each side)
-constexpr int NTH = 128;             // conv block: 4 warps
+constexpr int NTH = 192;             // conv block: 4 epilogue warps, a TMA warp, an MMA warp
 constexpr long long WAIT_LIMIT = 1ll << 26;
 
 __device__ __forceinline__ unsigned smem_u32(const void *p) {
     return static_cast<unsigned>(__cvta_generic_to_shared(p));
 }
 
-__device__ __forceinline__ void mbar_init(unsigned long long *bar) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)) : "memory");
+__device__ __forceinline__ void mbar_init(unsigned long long *bar, unsigned count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count)
+                 : "memory");
 }
 
-__device__ __forceinline__ bool mbar_wait(unsigned long long *bar, unsigned phase) {
+// Poll the phase with an iteration limit, or until another role of the block has given up.
+__device__ __forceinline__ bool mbar_wait(unsigned long long *bar, unsigned phase, const int *stop) {
     for (long long i = 0; i < WAIT_LIMIT; ++i) {
+        if (stop && (i & 1023) == 1023 && *(const volatile int *)stop) return false;
         unsigned done;
         asm volatile(
             "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;"
@@ -65,14 +67,24 @@ __device__ __forceinline__ void tma_load_4d(void *dst, const CUtensorMap *tm, in
         : "memory");
 }
 
+// arrives on the barrier when every MMA issued so far by this thread is complete
+__device__ __forceinline__ void commit(unsigned long long *bar) {
+    asm volatile(
+        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
+        : "memory");
+}
+
 // Shared-memory matrix descriptor (tcgen05): start, leading-dimension byte offset (between
-// core matrices along K), stride byte offset (between 8-row groups along M/N), no swizzle.
-__device__ __forceinline__ unsigned long long sdesc(unsigned addr, unsigned lbo, unsigned sbo) {
+// core matrices along K; unused by a swizzled operand as wide as its swizzle), stride byte
+// offset (between 8-row groups along M/N), swizzle (0 none, 4 64-byte, 6 32-byte).
+__device__ __forceinline__ unsigned long long sdesc(unsigned addr, unsigned lbo, unsigned sbo,
+                                                    unsigned swizzle) {
     unsigned long long d = 0;
     d |= (unsigned long long)((addr >> 4) & 0x3FFFu);
     d |= (unsigned long long)((lbo >> 4) & 0x3FFFu) << 16;
     d |= (unsigned long long)((sbo >> 4) & 0x3FFFu) << 32;
     d |= 1ull << 46;  // descriptor version of the 5th-generation tensor cores
+    d |= (unsigned long long)swizzle << 61;
     return d;
 }
 
@@ -126,54 +138,102 @@ __device__ __forceinline__ void store_row<float>(float *dst, const float *v, int
         *reinterpret_cast<float4 *>(dst + c) = make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]);
 }
 
+// a pixel of N channels in whole 32-byte sectors (dst 32-byte aligned)
+__device__ __forceinline__ void st32(void *dst, const unsigned *r) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(r[0]),
+                 "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+                 : "memory");
+}
+
+template <int N>
+__device__ __forceinline__ void store_pixel(__nv_bfloat16 *dst, const float *v) {
+#pragma unroll
+    for (int c = 0; c < N; c += 16) {
+        unsigned r[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const __nv_bfloat162 h = __floats2bfloat162_rn(v[c + 2 * i], v[c + 2 * i + 1]);
+            r[i] = *reinterpret_cast<const unsigned *>(&h);
+        }
+        st32(dst + c, r);
+    }
+}
+
+template <int N>
+__device__ __forceinline__ void store_pixel(float *dst, const float *v) {
+#pragma unroll
+    for (int c = 0; c < N; c += 8) {
+        unsigned r[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) r[i] = __float_as_uint(v[c + i]);
+        st32(dst + c, r);
+    }
+}
+
 // y[img][h][w][co] = act(b[co] + sum_taps sum_ci x[img][h+dy-1][w+dx-1][ci] W[tap][ci][co])
 // wprep: [9][CIN/8][COUT][8] BF16 (the canonical K-major B operand per tap).
 //
-// A CTA owns a strip (one image, 128 columns, all H rows) at a time and marches down it: input
-// rows arrive by TMA in a ring of RROWS slots (each row once per strip), so output row y
-// takes its three taps' rows from slots y - 1, y, y + 1.  One thread waits for the rows,
-// issues the 9 x CIN/16 MMAs of row y into one of two TMEM accumulators and commits; the
-// four warps meanwhile drain row y - 1 from the other accumulator (bias, ReLU, scale,
-// store).  When row y - 1's MMAs are complete its oldest input slot is refilled, RROWS - 3
-// rows ahead of use.  Every wait is bounded; on a timeout the CTA records the error, lets
-// its copies and MMAs in flight finish and leaves.
+// A unit of work is 128 columns of `rows` rows of one image; a CTA takes units in turn.  Three
+// roles share its rows without a block-wide barrier:
+//   warp 4 (one thread) stages input rows by TMA in a ring of RROWS slots, across unit ends,
+//   warp 5 (one thread) issues the 9 x CIN/16 MMAs of a row into one of two accumulators,
+//   warps 0 .. 3 drain it (bias, ReLU, scale, store) while the next row's MMAs run.
+// A slot is freed by the commit of the last row that reads it.  Every wait is bounded; on a
+// timeout the roles leave their loops and the copies and MMAs in flight are waited for.
+//
+// What bounds it: activation traffic (96 flop/B).  An input row is one TMA box of whole pixels
+// (CIN * 2 bytes) in the swizzle of that width: boxes of one 8-channel chunk each, which the
+// unswizzled layout needs, are CIN/8 times as many 16-byte requests and were the limit, with the
+// barrier per row: the network on 304 images of 121 x 401 took 2.75 ms, 2.07 ms so.  A tap is the row shifted by dx pixels: the slots start on the swizzle's
+// period, so the descriptor's start address moves by whole pixels with base offset 0.
 constexpr int RROWS = 6;
+constexpr int NEPI = 4;   // epilogue warps (one TMEM lane quarter each)
 
 template <int CIN, int COUT>
 struct ConvGeom {
-    static constexpr int NCH = CIN / 8;
-    static constexpr int RB = (PW * 16 + 127) / 128 * 128;   // one 8-channel row chunk (2176 B)
-    static constexpr int SLOT = NCH * RB;                      // one staged input row
+    static constexpr int RB = CIN * 2;                        // bytes of a pixel
+    static constexpr int PERIOD = 8 * RB;                     // the swizzle's period: 8 pixels
+    static constexpr int SLOT = (PW * RB + PERIOD - 1) / PERIOD * PERIOD;   // a staged input row
     static constexpr int RING = RROWS * SLOT;
-    static constexpr int WTAP = CIN * COUT * 2;                // one tap's weights
+    static constexpr int WTAP = CIN * COUT * 2;               // one tap's weights
     static constexpr int SMEM = (RING + 1023) / 1024 * 1024 + 9 * WTAP + 1024;
     static constexpr int TCOLS = 2 * COUT <= 32 ? 32 : (2 * COUT <= 64 ? 64 : 128);
 };
 
 template <int CIN, int COUT, bool RELU, typename OUT>
-__global__ void __launch_bounds__(NTH) conv3x3_tc_kernel(const __grid_constant__ CUtensorMap in_map,
+__global__ void __launch_bounds__(NTH, CIN == 16 ? 4 : 3) conv3x3_tc_kernel(const __grid_constant__ CUtensorMap in_map,
                                                          const __nv_bfloat16 *__restrict__ wprep,
                                                          const float *__restrict__ bias,
                                                          OUT *__restrict__ out, int nimg, int H,
-                                                         int W, int *dev_err, ConvEpi epi) {
+                                                         int W, int rows, int *dev_err, ConvEpi epi) {
     using Gm = ConvGeom<CIN, COUT>;
-    constexpr int NCH = Gm::NCH, RB = Gm::RB, SLOT = Gm::SLOT;
+    constexpr int RB = Gm::RB, SLOT = Gm::SLOT;
     constexpr unsigned IDESC = idesc_bf16(TM, COUT);
+    constexpr unsigned SWZ = CIN == 32 ? 4u : 6u;   // 64- or 32-byte swizzle
+    static_assert(CIN == 32 || CIN == 16, "a pixel is one swizzle row");
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    // align the dynamic shared memory base at run time (TMA destinations need 128 bytes)
-    unsigned char *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    unsigned char *ring = smem;
-    unsigned char *wsm = smem + (Gm::RING + 1023) / 1024 * 1024;
-    __shared__ __align__(8) unsigned long long bar_full[RROWS], bar_mma[2];
+    // the swizzle's period needs an aligned base
+    unsigned char *ring = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    unsigned char *wsm = ring + (Gm::RING + 1023) / 1024 * 1024;
+    // full: a slot's row has landed; empty: its last reader's MMAs are done; mma: an
+    // accumulator is complete; drained: every epilogue warp has read it
+    __shared__ __align__(8) unsigned long long full[RROWS], empty[RROWS], mma[2], drained[2];
     __shared__ unsigned tmem_base;
+    __shared__ int stop;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     for (int i = tid; i < 9 * Gm::WTAP / 16; i += NTH)
         reinterpret_cast<uint4 *>(wsm)[i] = reinterpret_cast<const uint4 *>(wprep)[i];
     if (tid == 0) {
-        for (int k = 0; k < RROWS; ++k) mbar_init(&bar_full[k]);
-        mbar_init(&bar_mma[0]);
-        mbar_init(&bar_mma[1]);
+        stop = 0;
+        for (int k = 0; k < RROWS; ++k) {
+            mbar_init(&full[k], 1);
+            mbar_init(&empty[k], 1);
+        }
+        for (int k = 0; k < 2; ++k) {
+            mbar_init(&mma[k], 1);
+            mbar_init(&drained[k], NEPI);
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     // the weights were written through the generic proxy; the tensor core reads them
@@ -191,133 +251,141 @@ __global__ void __launch_bounds__(NTH) conv3x3_tc_kernel(const __grid_constant__
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const unsigned tmem = tmem_base;
-    const int tiles_x = (W + TM - 1) / TM;
-    const long long nstrips = (long long)nimg * tiles_x;
-    const int nin = H + 2;            // input rows -1 .. H of a strip
-    unsigned seq_in = 0;              // input rows staged by this CTA before the current strip
-    unsigned seq_out = 0;             // output rows computed before the current strip
-    int issued = 0;                   // input rows of the current strip issued so far
-    int mma_open = -1;                // output row whose MMAs may still be in flight
-    bool late = false;
-    // input row j of the strip: slot (seq_in + j) % RROWS, completed phase parity
-    auto slot_of = [&](int j) { return (seq_in + (unsigned)j) % RROWS; };
-    auto par_in = [&](int j) { return ((seq_in + (unsigned)j) / RROWS) & 1u; };
-    for (long long st = blockIdx.x; st < nstrips; st += gridDim.x) {
-        const int tx = int(st % tiles_x), img = int(st / tiles_x);
-        const int x0 = tx * TM;
-        auto issue = [&](int j) {   // thread 0: stage input row j - 1
-            const unsigned k = slot_of(j);
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(
-                             smem_u32(&bar_full[k])),
-                         "r"((unsigned)(NCH * PW * 16))
-                         : "memory");
-#pragma unroll
-            for (int c = 0; c < NCH; ++c)
-                tma_load_4d(ring + k * SLOT + c * RB, &in_map, 8 * c, x0 - 1, j - 1, img,
-                            &bar_full[k]);
-        };
-        issued = min(nin, RROWS);
-        if (tid == 0)
-            for (int j = 0; j < issued; ++j) issue(j);
-        const float sc = epi.oscale ? epi.oscale[img] : 1.0f;   // per-image output factor
-        float isc = 1.0f;                                        // per-image input factor
-        if (epi.irms) {
-            const float r = epi.irms[img];
-            isc = r > 0.0f ? 1.0f / r : 0.0f;
+    const int tiles_x = (W + TM - 1) / TM, nseg = (H + rows - 1) / rows;
+    const long long nunits = (long long)nimg * nseg * tiles_x;
+    auto wait = [&](unsigned long long *bar, unsigned phase) {
+        const bool ok = mbar_wait(bar, phase, &stop);
+        if (!ok) {
+            *(volatile int *)&stop = 1;
+            atomicExch(dev_err, DEV_ERR_TMA_TIMEOUT);
         }
-        auto epilogue = [&](int y, unsigned o) {
-            float v[COUT];
-            tmem_ld<COUT>(tmem + ((unsigned)(warp * 32) << 16) + (o & 1u) * COUT, v);
-            const int px = x0 + warp * 32 + lane;
-            if (px < W) {
-#pragma unroll
-                for (int c = 0; c < COUT; ++c) {
-                    float a = v[c] * isc + (bias ? bias[c] : 0.0f);
-                    v[c] = sc * (RELU ? fmaxf(a, 0.0f) : a);
-                }
-                if (epi.nchw) {   // planes [img][c][H][W]: coalesced along px per channel
-                    OUT *o0 = out + ((long long)img * COUT * H + y) * W + px;
-#pragma unroll
-                    for (int c = 0; c < COUT; ++c) o0[(long long)c * H * W] = OUT(v[c]);
-                } else {
-                    store_row<OUT>(out + (((long long)img * H + y) * W + px) * COUT, v, COUT);
+        return ok;
+    };
+    // unit u: columns x0 .. x0 + 127, rows y0 .. y0 + ny - 1 of image img; its input row j is
+    // row y0 + j - 1 of the image, j = 0 .. ny + 1
+    int x0 = 0, y0 = 0, ny = 0, img = 0;
+    auto take = [&](long long u) {
+        x0 = int(u % tiles_x) * TM;
+        const long long v = u / tiles_x;
+        y0 = int(v % nseg) * rows;
+        img = int(v / nseg);
+        ny = min(rows, H - y0);
+    };
+    if (warp == NEPI) {
+        if (lane == 0) {
+            unsigned g = 0;   // input rows staged so far
+            bool ok = true;
+            for (long long u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
+                take(u);
+                for (int j = 0; j < ny + 2; ++j, ++g) {
+                    const unsigned k = g % RROWS;
+                    if (g >= RROWS && !(ok = wait(&empty[k], (g / RROWS - 1) & 1u))) break;
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(
+                                     smem_u32(&full[k])),
+                                 "r"((unsigned)(PW * RB))
+                                 : "memory");
+                    tma_load_4d(ring + k * SLOT, &in_map, 0, x0 - 1, y0 + j - 1, img, &full[k]);
                 }
             }
-        };
-        for (int y = 0; y < H; ++y) {
-            const unsigned o = seq_out + (unsigned)y;
-            if (tid == 0) {
-                bool ok = true;
+            // (after a timeout the rows in flight may have had no reader)
+            for (unsigned i = g > RROWS ? g - RROWS : 0; i < g; ++i)
+                mbar_wait(&full[i % RROWS], (i / RROWS) & 1u, nullptr);
+        }
+    } else if (warp == NEPI + 1) {
+        if (lane == 0) {
+            unsigned g = 0, o = 0;   // input rows of the units before, output rows issued
+            unsigned done = 0;       // input rows whose slots have been handed to a commit
+            bool ok = true;
+            const unsigned wb = smem_u32(wsm), rb = smem_u32(ring);
+            for (long long u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
+                take(u);
+                for (int y = 0; y < ny; ++y, ++o) {
+                    for (int d = y == 0 ? 0 : 2; d < 3 && ok; ++d) {
+                        const unsigned r = g + y + d;
+                        ok = wait(&full[r % RROWS], (r / RROWS) & 1u);
+                    }
+                    if (ok && o >= 2) ok = wait(&drained[o & 1u], ((o >> 1) - 1) & 1u);
+                    if (!ok) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const unsigned acc_addr = tmem + (o & 1u) * COUT;
 #pragma unroll
-                for (int d = 0; d < 3; ++d) ok &= mbar_wait(&bar_full[slot_of(y + d)], par_in(y + d));
-                late |= !ok;
+                    for (int tap = 0; tap < 9; ++tap) {
+                        const int dy = tap / 3, dx = tap % 3;
+                        const unsigned pa = rb + ((g + y + dy) % RROWS) * SLOT;
+#pragma unroll
+                        for (int ks = 0; ks < CIN / 16; ++ks) {
+                            const unsigned long long da =
+                                sdesc(pa + dx * RB + ks * 32, 16, Gm::PERIOD, SWZ);
+                            const unsigned long long db =
+                                sdesc(wb + tap * Gm::WTAP + ks * 2 * COUT * 16, COUT * 16, 128, 0);
+                            const unsigned acc = (tap | ks) ? 1u : 0u;
+                            asm volatile(
+                                "{ .reg .pred p; setp.ne.u32 p, %4, 0;"
+                                " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p; }" ::"r"(
+                                    acc_addr),
+                                "l"(da), "l"(db), "r"(IDESC), "r"(acc)
+                                : "memory");
+                        }
+                    }
+                    commit(&mma[o & 1u]);
+                    // input row y has no later reader; with the unit's last row, all of them
+                    for (const unsigned e = g + y + (y == ny - 1 ? 3 : 1); done < e; ++done)
+                        commit(&empty[done % RROWS]);
+                }
+                g += (unsigned)ny + 2;
+            }
+            // every commit has arrived before the barriers and the TMEM go
+            for (unsigned i = done > RROWS ? done - RROWS : 0; i < done; ++i)
+                mbar_wait(&empty[i % RROWS], (i / RROWS) & 1u, nullptr);
+            if (o > 0) mbar_wait(&mma[(o - 1) & 1u], ((o - 1) >> 1) & 1u, nullptr);
+        }
+    } else {
+        unsigned o = 0;
+        bool ok = true;
+        for (long long u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
+            take(u);
+            const float sc = epi.oscale ? epi.oscale[img] : 1.0f;   // per-image output factor
+            float isc = 1.0f;                                        // per-image input factor
+            if (epi.irms) {
+                const float r = epi.irms[img];
+                isc = r > 0.0f ? 1.0f / r : 0.0f;
+            }
+            const int px = x0 + tid;
+            for (int y = 0; y < ny; ++y, ++o) {
+                ok = __all_sync(0xffffffffu, wait(&mma[o & 1u], (o >> 1) & 1u));
+                if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const unsigned wb = smem_u32(wsm), acc_addr = tmem + (o & 1u) * COUT;
+                float v[COUT];
+                tmem_ld<COUT>(tmem + ((unsigned)(warp * 32) << 16) + (o & 1u) * COUT, v);
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0)
+                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(
+                                     smem_u32(&drained[o & 1u]))
+                                 : "memory");
+                if (px < W) {
 #pragma unroll
-                for (int tap = 0; tap < 9; ++tap) {
-                    const int dy = tap / 3, dx = tap % 3;
-                    const unsigned pa = smem_u32(ring + slot_of(y + dy) * SLOT);
+                    for (int c = 0; c < COUT; ++c) {
+                        const float a = v[c] * isc + (bias ? bias[c] : 0.0f);
+                        v[c] = sc * (RELU ? fmaxf(a, 0.0f) : a);
+                    }
+                    if (epi.nchw) {   // planes [img][c][H][W]: coalesced along px per channel
+                        OUT *q = out + ((long long)img * COUT * H + y0 + y) * W + px;
 #pragma unroll
-                    for (int ks = 0; ks < CIN / 16; ++ks) {
-                        const unsigned long long da = sdesc(pa + ks * 2 * RB + dx * 16, RB, 128);
-                        const unsigned long long db =
-                            sdesc(wb + tap * Gm::WTAP + ks * 2 * COUT * 16, COUT * 16, 128);
-                        const unsigned acc = (tap | ks) ? 1u : 0u;
-                        asm volatile(
-                            "{ .reg .pred p; setp.ne.u32 p, %4, 0;"
-                            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p; }" ::"r"(
-                                acc_addr),
-                            "l"(da), "l"(db), "r"(IDESC), "r"(acc)
-                            : "memory");
+                        for (int c = 0; c < COUT; ++c) q[(long long)c * H * W] = OUT(v[c]);
+                    } else {
+                        OUT *q = out + (((long long)img * H + y0 + y) * W + px) * COUT;
+                        if (epi.wide)
+                            store_pixel<COUT>(q, v);
+                        else
+                            store_row<OUT>(q, v, COUT);
                     }
                 }
-                asm volatile(
-                    "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                        smem_u32(&bar_mma[o & 1u]))
-                    : "memory");
+                __syncwarp();
             }
-            mma_open = y;
-            if (y >= 1) {
-                // row y - 1: its MMAs are complete once its commit arrives
-                late |= !mbar_wait(&bar_mma[(o - 1) & 1u], ((o - 1) >> 1) & 1u);
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                epilogue(y - 1, o - 1);
-                // input row y - 2 (sequence j = y - 1) had its last reader in row y - 1
-                if (tid == 0)
-                    while (issued < nin && issued <= y - 1 + RROWS) issue(issued++);
-                else
-                    issued = min(nin, max(issued, y + RROWS));
-            }
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            if (__syncthreads_or(late)) goto timeout;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        }
-        {
-            const unsigned o = seq_out + (unsigned)(H - 1);
-            late |= !mbar_wait(&bar_mma[o & 1u], (o >> 1) & 1u);
-            mma_open = -1;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            epilogue(H - 1, o);
-        }
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        if (__syncthreads_or(late)) goto timeout;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        seq_in += (unsigned)nin;
-        seq_out += (unsigned)H;
-    }
-    goto done;
-timeout:
-    // let the copies and the MMAs in flight finish before the TMEM and shared memory go
-    if (tid == 0) {
-        atomicExch(dev_err, DEV_ERR_TMA_TIMEOUT);
-        for (int j = max(0, issued - RROWS); j < issued; ++j) mbar_wait(&bar_full[slot_of(j)], par_in(j));
-        if (mma_open >= 0) {
-            const unsigned o = seq_out + (unsigned)mma_open;
-            mbar_wait(&bar_mma[o & 1u], (o >> 1) & 1u);
         }
     }
-    __syncthreads();
-done:
+    __syncwarp();
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0)
@@ -869,12 +937,29 @@ cudaError_t make_act_map(CUtensorMap *tm, const void *base, int C_, int W, int H
     const cuuint64_t dims[4] = {(cuuint64_t)C_, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)n};
     const cuuint64_t strides[3] = {(cuuint64_t)C_ * 2, (cuuint64_t)W * C_ * 2,
                                    (cuuint64_t)H * W * C_ * 2};
-    const cuuint32_t box[4] = {8, (cuuint32_t)PW, 1, 1};
+    const cuuint32_t box[4] = {(cuuint32_t)C_, (cuuint32_t)PW, 1, 1};
     const cuuint32_t es[4] = {1, 1, 1, 1};
     CUresult r = enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(base), dims, strides,
-                     box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                     box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                     C_ == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
                      CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+// Rows of a unit (even): the split of the strips that costs the fewest rows in a row for one CTA,
+// counting the two halo rows and about four rows' time to fill the pipeline.  Whole strips leave
+// a last round part-filled: 1216 strips on 456 CTAs take three rounds of 121 rows, thirds of them
+// eight of 42.
+static int unit_rows(int H, long long strips, long long slots) {
+    int best = H + (H & 1);
+    long long cost = -1;
+    for (int n = 1; n <= std::max(1, H / 16); ++n) {
+        const int rows = 2 * ((H + 2 * n - 1) / (2 * n));
+        const long long units = strips * ((H + rows - 1) / rows);
+        const long long c = (units + slots - 1) / slots * (rows + 6);
+        if (cost < 0 || c < cost) cost = c, best = rows;
+    }
+    return best;
 }
 
 template <int CIN, int COUT, bool RELU, typename OUT>
@@ -911,9 +996,13 @@ cudaError_t conv_launch(const void *in, const __nv_bfloat16 *wprep, const float 
         return cudaSuccess;
     });
     if (e != cudaSuccess) return e;
-    const long long strips = (long long)nimg * ((W + TM - 1) / TM);
-    const int grid = (int)std::min<long long>(strips, (long long)nsm * per_sm);
-    kern<<<grid, NTH, Gm::SMEM, st>>>(tm, wprep, bias, out, nimg, H, W, dev_err, epi);
+    const long long strips = (long long)nimg * ((W + TM - 1) / TM), slots = (long long)nsm * per_sm;
+    const int rows = unit_rows(H, strips, slots);
+    const long long units = strips * ((H + rows - 1) / rows);
+    const int grid = (int)std::min(units, slots);
+    ConvEpi ep = epi;
+    ep.wide = reinterpret_cast<uintptr_t>(out) % 32 == 0;
+    kern<<<grid, NTH, Gm::SMEM, st>>>(tm, wprep, bias, out, nimg, H, W, rows, dev_err, ep);
     return cudaGetLastError();
 }
 
