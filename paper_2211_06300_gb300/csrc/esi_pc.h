@@ -46,8 +46,12 @@ struct ConvEpi {
     const float *irms = nullptr;     // per-image input RMS: the accumulator is divided by it
     int wide = 0;                    // (set by the launch) the output is 32-byte aligned
     int nchw = 0;                    // output planes [img][c][H][W] instead of channels-last
+    __nv_bfloat16 *pool = nullptr;   // also the output's 2 x 2 averages (zero fill at odd edges)
+    const __nv_bfloat16 *up = nullptr;   // UP: the half-resolution summand of the input
+    __nv_bfloat16 *u_out = nullptr;      // UP: the sum, where the weight gradient wants it
 };
-template <int CIN, int COUT, bool RELU, typename OUT>
+// UP: the input is in + up(epi.up), nearest-neighbour upsampled, summed in BF16
+template <int CIN, int COUT, bool RELU, typename OUT, bool UP = false>
 cudaError_t conv_launch(const void *in, const __nv_bfloat16 *wprep, const float *bias, OUT *out,
                         int nimg, int H, int W, int *dev_err, int nsm, cudaStream_t st,
                         const ConvEpi &epi = ConvEpi());
@@ -61,10 +65,6 @@ cudaError_t wprep_launch(const float *W, __nv_bfloat16 *out, int cin, int cout, 
 cudaError_t pack_launch(const float *r, const float *ipb2, __nv_bfloat16 *img, int ns, int nt,
                         int nz, int nx, int px, long long sst, int scale_by_map, int dense,
                         cudaStream_t st);
-cudaError_t pool_launch(const __nv_bfloat16 *in, __nv_bfloat16 *out, long long n, int H, int W,
-                        cudaStream_t st);
-cudaError_t upadd_launch(const __nv_bfloat16 *coarse, const __nv_bfloat16 *skip,
-                         __nv_bfloat16 *out, long long n, int H, int W, cudaStream_t st);
 cudaError_t mask_launch(float *g, const __nv_bfloat16 *act, __nv_bfloat16 *gb, long long n,
                         cudaStream_t st);
 cudaError_t pool_bwd_launch(float *gf, const float *gc, long long n, int H, int W, cudaStream_t st);

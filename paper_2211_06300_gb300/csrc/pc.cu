@@ -146,20 +146,6 @@ __device__ __forceinline__ void st32(void *dst, const unsigned *r) {
 }
 
 template <int N>
-__device__ __forceinline__ void store_pixel(__nv_bfloat16 *dst, const float *v) {
-#pragma unroll
-    for (int c = 0; c < N; c += 16) {
-        unsigned r[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const __nv_bfloat162 h = __floats2bfloat162_rn(v[c + 2 * i], v[c + 2 * i + 1]);
-            r[i] = *reinterpret_cast<const unsigned *>(&h);
-        }
-        st32(dst + c, r);
-    }
-}
-
-template <int N>
 __device__ __forceinline__ void store_pixel(float *dst, const float *v) {
 #pragma unroll
     for (int c = 0; c < N; c += 8) {
@@ -186,6 +172,13 @@ __device__ __forceinline__ void store_pixel(float *dst, const float *v) {
 // unswizzled layout needs, are CIN/8 times as many 16-byte requests and were the limit, with the
 // barrier per row: the network on 304 images of 121 x 401 took 2.75 ms, 2.07 ms so.  A tap is the row shifted by dx pixels: the slots start on the swizzle's
 // period, so the descriptor's start address moves by whole pixels with base offset 0.
+//
+// Pooling and the decoder's upsample-add are part of the convolutions around them: with epi.pool
+// the epilogue keeps an even row's pixels and writes the 2 x 2 averages with the odd one; with UP
+// the input is epi.up (half the resolution, nearest) + the staged skip row, added in its slot by
+// warps 0 .. 3 one row ahead of the MMAs (`ready` in the place of `full`).  As passes of their own
+// they moved 64 + 16 and 64 + 16 + 64 bytes a pixel and the decoder read 64 again: the same network
+2.07 -> 1.67 ms (first layer with its pooling 428 us, 3.7 TB/s; last one with its sum 568 us).
 constexpr int RROWS = 6;
 constexpr int NEPI = 4;   // epilogue warps (one TMEM lane quarter each)
 
@@ -200,7 +193,44 @@ struct ConvGeom {
     static constexpr int TCOLS = 2 * COUT <= 32 ? 32 : (2 * COUT <= 64 ? 64 : 128);
 };
 
-template <int CIN, int COUT, bool RELU, typename OUT>
+// The 2 x 2 average of a pixel pair's two rows (b zero beyond the grid): the even lane of the pair
+// has channels 0 .. 15, the odd lane 16 .. 31.  a, b: this lane's pixel, 32 BF16 channels; r: the
+// lane's half of the averages.
+__device__ __forceinline__ void pool_pair(const unsigned *a, const unsigned *b, bool odd, unsigned *r) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        unsigned c[4];   // left and right pixel of the upper row, then of the lower one
+        const unsigned ar = __shfl_xor_sync(0xffffffffu, odd ? a[i] : a[8 + i], 1);
+        const unsigned br = __shfl_xor_sync(0xffffffffu, odd ? b[i] : b[8 + i], 1);
+        c[0] = odd ? ar : a[i], c[1] = odd ? a[8 + i] : ar;
+        c[2] = odd ? br : b[i], c[3] = odd ? b[8 + i] : br;
+        float2 acc = make_float2(0.0f, 0.0f);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&c[k]));
+            acc.x += f.x;
+            acc.y += f.y;
+        }
+        const __nv_bfloat162 h = __floats2bfloat162_rn(acc.x * 0.25f, acc.y * 0.25f);
+        r[i] = *reinterpret_cast<const unsigned *>(&h);
+    }
+}
+
+// eight BF16 sums, rounded once
+__device__ __forceinline__ uint4 add8(const uint4 &a, const uint4 &b) {
+    uint4 q;
+    const __nv_bfloat162 *ha = reinterpret_cast<const __nv_bfloat162 *>(&a);
+    const __nv_bfloat162 *hb = reinterpret_cast<const __nv_bfloat162 *>(&b);
+    __nv_bfloat162 *hq = reinterpret_cast<__nv_bfloat162 *>(&q);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float2 fa = __bfloat1622float2(ha[k]), fb = __bfloat1622float2(hb[k]);
+        hq[k] = __floats2bfloat162_rn(fa.x + fb.x, fa.y + fb.y);
+    }
+    return q;
+}
+
+template <int CIN, int COUT, bool RELU, typename OUT, bool UP>
 __global__ void __launch_bounds__(NTH, CIN == 16 ? 4 : 3) conv3x3_tc_kernel(const __grid_constant__ CUtensorMap in_map,
                                                          const __nv_bfloat16 *__restrict__ wprep,
                                                          const float *__restrict__ bias,
@@ -218,6 +248,7 @@ __global__ void __launch_bounds__(NTH, CIN == 16 ? 4 : 3) conv3x3_tc_kernel(cons
     // full: a slot's row has landed; empty: its last reader's MMAs are done; mma: an
     // accumulator is complete; drained: every epilogue warp has read it
     __shared__ __align__(8) unsigned long long full[RROWS], empty[RROWS], mma[2], drained[2];
+    __shared__ __align__(8) unsigned long long ready[RROWS];   // UP: the sum is in the slot
     __shared__ unsigned tmem_base;
     __shared__ int stop;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -229,6 +260,7 @@ __global__ void __launch_bounds__(NTH, CIN == 16 ? 4 : 3) conv3x3_tc_kernel(cons
         for (int k = 0; k < RROWS; ++k) {
             mbar_init(&full[k], 1);
             mbar_init(&empty[k], 1);
+            mbar_init(&ready[k], NEPI);
         }
         for (int k = 0; k < 2; ++k) {
             mbar_init(&mma[k], 1);
@@ -302,7 +334,7 @@ __global__ void __launch_bounds__(NTH, CIN == 16 ? 4 : 3) conv3x3_tc_kernel(cons
                 for (int y = 0; y < ny; ++y, ++o) {
                     for (int d = y == 0 ? 0 : 2; d < 3 && ok; ++d) {
                         const unsigned r = g + y + d;
-                        ok = wait(&full[r % RROWS], (r / RROWS) & 1u);
+                        ok = wait(UP ? &ready[r % RROWS] : &full[r % RROWS], (r / RROWS) & 1u);
                     }
                     if (ok && o >= 2) ok = wait(&drained[o & 1u], ((o >> 1) - 1) & 1u);
                     if (!ok) break;
@@ -340,10 +372,62 @@ __global__ void __launch_bounds__(NTH, CIN == 16 ? 4 : 3) conv3x3_tc_kernel(cons
             if (o > 0) mbar_wait(&mma[(o - 1) & 1u], ((o - 1) >> 1) & 1u, nullptr);
         }
     } else {
-        unsigned o = 0;
+        unsigned o = 0, g = 0;   // output rows, input rows of the units before
         bool ok = true;
+        // UP: a thread adds the 16-byte pieces tid + 128 i of a row (130 pixels of four pieces;
+        // the 64-byte swizzle of a pixel's pieces follows bits 1, 2 of its number, the same for
+        // all i).  Two rows share the coarse row held in cr.
+        constexpr int NP = UP ? (PW * 4 + 127) / 128 : 1;
+        const int piece = (tid & 3) ^ ((tid >> 3) & 3);
+        uint4 cr[NP];
+        int crow = -1;
+        auto coarse = [&](int cy) {
+            const __nv_bfloat16 *c0 =
+                epi.up + (((long long)img * ((H + 1) / 2) + cy) * ((W + 1) / 2)) * 32 + piece * 8;
+#pragma unroll
+            for (int i = 0; i < NP; ++i) {
+                const int p = (tid >> 2) + 32 * i, x = x0 - 1 + p;
+                if (p < PW && x >= 0 && x < W)
+                    cr[i] = __ldg(reinterpret_cast<const uint4 *>(c0 + (x >> 1) * 32));
+            }
+            crow = cy;
+        };
+        auto sum_row = [&](int j) {
+            const int gy = y0 + j - 1;
+            const unsigned k = (g + (unsigned)j) % RROWS;
+            const bool in = gy >= 0 && gy < H;
+            if (in && crow != gy >> 1) coarse(gy >> 1);
+            ok = __all_sync(0xffffffffu, wait(&full[k], ((g + (unsigned)j) / RROWS) & 1u));
+            if (!ok) return;
+            if (in) {
+                uint4 *sl = reinterpret_cast<uint4 *>(ring + k * SLOT);
+#pragma unroll
+                for (int i = 0; i < NP; ++i) {
+                    const int p = (tid >> 2) + 32 * i, x = x0 - 1 + p;
+                    if (p < PW && x >= 0 && x < W) {
+                        const uint4 q = add8(cr[i], sl[tid + 128 * i]);
+                        sl[tid + 128 * i] = q;
+                        if (epi.u_out && p >= 1 && p <= TM && j >= 1 && j <= ny)
+                            *reinterpret_cast<uint4 *>(
+                                epi.u_out + (((long long)img * H + gy) * W + x) * 32 + piece * 8) = q;
+                    }
+                }
+                // the next row's coarse values arrive while a row is drained
+                if ((gy & 1) && gy + 1 < H && j <= ny) coarse((gy + 1) >> 1);
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&ready[k]))
+                             : "memory");
+        };
         for (long long u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
             take(u);
+            if constexpr (UP) {
+                crow = -1;
+                for (int j = 0; j < 3 && ok; ++j) sum_row(j);
+                if (!ok) break;
+            }
             const float sc = epi.oscale ? epi.oscale[img] : 1.0f;   // per-image output factor
             float isc = 1.0f;                                        // per-image input factor
             if (epi.irms) {
@@ -351,7 +435,13 @@ __global__ void __launch_bounds__(NTH, CIN == 16 ? 4 : 3) conv3x3_tc_kernel(cons
                 isc = r > 0.0f ? 1.0f / r : 0.0f;
             }
             const int px = x0 + tid;
+            unsigned even[sizeof(OUT) == 2 && !UP ? COUT / 2 : 1];   // the even row, for pooling
+            (void)even;
             for (int y = 0; y < ny; ++y, ++o) {
+                if constexpr (UP) {
+                    if (y + 1 < ny) sum_row(y + 3);
+                    if (!ok) break;
+                }
                 ok = __all_sync(0xffffffffu, wait(&mma[o & 1u], (o >> 1) & 1u));
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -363,26 +453,54 @@ __global__ void __launch_bounds__(NTH, CIN == 16 ? 4 : 3) conv3x3_tc_kernel(cons
                     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(
                                      smem_u32(&drained[o & 1u]))
                                  : "memory");
-                if (px < W) {
 #pragma unroll
-                    for (int c = 0; c < COUT; ++c) {
-                        const float a = v[c] * isc + (bias ? bias[c] : 0.0f);
-                        v[c] = sc * (RELU ? fmaxf(a, 0.0f) : a);
+                for (int c = 0; c < COUT; ++c) {
+                    const float a = v[c] * isc + (bias ? bias[c] : 0.0f);
+                    v[c] = sc * (RELU ? fmaxf(a, 0.0f) : a);
+                }
+                OUT *q = out + (((long long)img * H + y0 + y) * W + px) * COUT;
+                if constexpr (sizeof(OUT) == 2) {
+                    unsigned pk[COUT / 2];
+#pragma unroll
+                    for (int c = 0; c < COUT / 2; ++c) {
+                        const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * c], v[2 * c + 1]);
+                        pk[c] = px < W ? *reinterpret_cast<const unsigned *>(&h) : 0u;
                     }
-                    if (epi.nchw) {   // planes [img][c][H][W]: coalesced along px per channel
-                        OUT *q = out + ((long long)img * COUT * H + y0 + y) * W + px;
+                    if (px < W) {
 #pragma unroll
-                        for (int c = 0; c < COUT; ++c) q[(long long)c * H * W] = OUT(v[c]);
+                        for (int c = 0; c < COUT / 2; c += 8) st32(q + 2 * c, pk + c);
+                    }
+                    if constexpr (!UP) {
+                        if (epi.pool) {   // y0 is even: the parity of y is the row's
+                            static_assert(COUT == 32, "a lane pair averages 16 channels each");
+                            if (!(y & 1)) {
+    #pragma unroll
+                                for (int c = 0; c < COUT / 2; ++c) even[c] = pk[c], pk[c] = 0u;
+                            }
+                            if ((y & 1) || y == ny - 1) {
+                                unsigned r[8];
+                                pool_pair(even, pk, lane & 1, r);
+                                if ((px & ~1) < W)
+                                    st32(epi.pool + (((long long)img * ((H + 1) / 2) + (y0 + y) / 2) *
+                                                         ((W + 1) / 2) + (px >> 1)) * COUT + 16 * (lane & 1),
+                                         r);
+                            }
+                        }
+                    }
+                } else if (px < W) {
+                    if (epi.nchw) {   // planes [img][c][H][W]: coalesced along px per channel
+                        OUT *qp = out + ((long long)img * COUT * H + y0 + y) * W + px;
+#pragma unroll
+                        for (int c = 0; c < COUT; ++c) qp[(long long)c * H * W] = OUT(v[c]);
+                    } else if (epi.wide) {
+                        store_pixel<COUT>(q, v);
                     } else {
-                        OUT *q = out + (((long long)img * H + y0 + y) * W + px) * COUT;
-                        if (epi.wide)
-                            store_pixel<COUT>(q, v);
-                        else
-                            store_row<OUT>(q, v, COUT);
+                        store_row<OUT>(q, v, COUT);
                     }
                 }
                 __syncwarp();
             }
+            g += (unsigned)ny + 2;
         }
     }
     __syncwarp();
@@ -524,64 +642,6 @@ __global__ void __launch_bounds__(256, 4) pack4_kernel(const float *r, const flo
                                              G / 2);
             }
         }
-    }
-}
-
-// 2 x 2 average pooling (zero fill at odd edges), BF16 channels-last, C = 32
-__global__ void pool_kernel(const __nv_bfloat16 *in, __nv_bfloat16 *out, long long n, int H, int W,
-                            int Ho, int Wo) {
-    const long long total = n * Ho * Wo * (C / 8);
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int ch = int(i % (C / 8));
-        const long long p = i / (C / 8);
-        const int x = int(p % Wo);
-        const long long r1 = p / Wo;
-        const int y = int(r1 % Ho);
-        const long long img = r1 / Ho;
-        float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        for (int a = 0; a < 2; ++a)
-            for (int b = 0; b < 2; ++b) {
-                const int iy = 2 * y + a, ix = 2 * x + b;
-                if (iy >= H || ix >= W) continue;
-                const uint4 q = *reinterpret_cast<const uint4 *>(in + ((img * H + iy) * W + ix) * C + ch * 8);
-                const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&q);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const float2 f = __bfloat1622float2(h[k]);
-                    acc[2 * k] += f.x;
-                    acc[2 * k + 1] += f.y;
-                }
-            }
-        for (int k = 0; k < 8; ++k) acc[k] *= 0.25f;
-        store_row<__nv_bfloat16>(out + p * C + ch * 8, acc, 8);
-    }
-}
-
-// out[h][w] = coarse[h/2][w/2] + skip[h][w]  (C = 32)
-__global__ void upadd_kernel(const __nv_bfloat16 *coarse, const __nv_bfloat16 *skip,
-                             __nv_bfloat16 *out, long long n, int H, int W, int Hc, int Wc) {
-    const long long total = n * H * W * (C / 8);
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int ch = int(i % (C / 8));
-        const long long p = i / (C / 8);
-        const int x = int(p % W);
-        const long long r1 = p / W;
-        const int y = int(r1 % H);
-        const long long img = r1 / H;
-        const uint4 a = *reinterpret_cast<const uint4 *>(coarse + ((img * Hc + y / 2) * Wc + x / 2) * C + ch * 8);
-        const uint4 b = *reinterpret_cast<const uint4 *>(skip + p * C + ch * 8);
-        const __nv_bfloat162 *ha = reinterpret_cast<const __nv_bfloat162 *>(&a);
-        const __nv_bfloat162 *hb = reinterpret_cast<const __nv_bfloat162 *>(&b);
-        float o[8];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const float2 fa = __bfloat1622float2(ha[k]), fb = __bfloat1622float2(hb[k]);
-            o[2 * k] = fa.x + fb.x;
-            o[2 * k + 1] = fa.y + fb.y;
-        }
-        store_row<__nv_bfloat16>(out + p * C + ch * 8, o, 8);
     }
 }
 
@@ -962,15 +1022,17 @@ static int unit_rows(int H, long long strips, long long slots) {
     return best;
 }
 
-template <int CIN, int COUT, bool RELU, typename OUT>
+template <int CIN, int COUT, bool RELU, typename OUT, bool UP>
 cudaError_t conv_launch(const void *in, const __nv_bfloat16 *wprep, const float *bias, OUT *out,
                         int nimg, int H, int W, int *dev_err, int nsm, cudaStream_t st,
                         const ConvEpi &epi) {
     using Gm = ConvGeom<CIN, COUT>;
+    const bool wide = reinterpret_cast<uintptr_t>(out) % 32 == 0;
+    if (sizeof(OUT) == 2 && !wide) return cudaErrorInvalidValue;   // (internal activations)
     CUtensorMap tm;
     cudaError_t e = make_act_map(&tm, in, CIN, W, H, nimg);
     if (e != cudaSuccess) return e;
-    auto kern = conv3x3_tc_kernel<CIN, COUT, RELU, OUT>;
+    auto kern = conv3x3_tc_kernel<CIN, COUT, RELU, OUT, UP>;
     static PerDevice cache;
     int per_sm = 0;
     e = per_device(cache, &per_sm, [kern](int *v) {
@@ -1001,20 +1063,21 @@ cudaError_t conv_launch(const void *in, const __nv_bfloat16 *wprep, const float 
     const long long units = strips * ((H + rows - 1) / rows);
     const int grid = (int)std::min(units, slots);
     ConvEpi ep = epi;
-    ep.wide = reinterpret_cast<uintptr_t>(out) % 32 == 0;
+    ep.wide = wide;
     kern<<<grid, NTH, Gm::SMEM, st>>>(tm, wprep, bias, out, nimg, H, W, rows, dev_err, ep);
     return cudaGetLastError();
 }
 
-#define CONV_INST(CI, CO, R, O)                                                                 \
-    template cudaError_t conv_launch<CI, CO, R, O>(const void *, const __nv_bfloat16 *,        \
-                                                   const float *, O *, int, int, int, int *,   \
-                                                   int, cudaStream_t, const ConvEpi &);
-CONV_INST(16, 32, true, __nv_bfloat16)
-CONV_INST(32, 32, true, __nv_bfloat16)
-CONV_INST(32, 16, false, float)
-CONV_INST(16, 32, false, float)
-CONV_INST(32, 32, false, float)
+#define CONV_INST(CI, CO, R, O, UP)                                                              \
+    template cudaError_t conv_launch<CI, CO, R, O, UP>(const void *, const __nv_bfloat16 *,     \
+                                                       const float *, O *, int, int, int, int *, \
+                                                       int, cudaStream_t, const ConvEpi &);
+CONV_INST(16, 32, true, __nv_bfloat16, false)
+CONV_INST(32, 32, true, __nv_bfloat16, false)
+CONV_INST(32, 32, true, __nv_bfloat16, true)
+CONV_INST(32, 16, false, float, true)
+CONV_INST(16, 32, false, float, false)
+CONV_INST(32, 32, false, float, false)
 #undef CONV_INST
 
 cudaError_t normalize_launch(const __nv_bfloat16 *x, float *rms, double *acc, __nv_bfloat16 *xn,
@@ -1053,20 +1116,6 @@ cudaError_t pack_launch(const float *r, const float *ipb2, __nv_bfloat16 *img, i
     }
     pack_kernel<<<std::min(nrow, 4096), 256, 0, st>>>(r, ipb2, img, ns, nt, ng, nz, nx, px, sst,
                                                          hc, wc, scale_by_map, dense);
-    return cudaGetLastError();
-}
-
-cudaError_t pool_launch(const __nv_bfloat16 *in, __nv_bfloat16 *out, long long n, int H, int W,
-                        cudaStream_t st) {
-    const int Ho = (H + 1) / 2, Wo = (W + 1) / 2;
-    pool_kernel<<<grid_for(n * Ho * Wo * (C / 8)), 256, 0, st>>>(in, out, n, H, W, Ho, Wo);
-    return cudaGetLastError();
-}
-
-cudaError_t upadd_launch(const __nv_bfloat16 *coarse, const __nv_bfloat16 *skip, __nv_bfloat16 *out,
-                         long long n, int H, int W, cudaStream_t st) {
-    upadd_kernel<<<grid_for(n * H * W * (C / 8)), 256, 0, st>>>(coarse, skip, out, n, H, W,
-                                                                (H + 1) / 2, (W + 1) / 2);
     return cudaGetLastError();
 }
 

@@ -158,22 +158,30 @@ cudaError_t pcnet_forward(PcNet *p, const __nv_bfloat16 *x, int n, float *y, cud
         x = p->xn.as<bf>();
     else
         e0.irms = p->rms.as<float>();   // conv(x / rms) = conv(x) / rms before the bias
+    e0.pool = p->p1.as<bf>();
     RET((conv_launch<G, C, true, bf>(x, wf(0), bias_of(p, 0), p->e1.as<bf>(), n, H[0], W[0], de, p->nsm, st, e0)));
-    RET(pool_launch(p->e1.as<bf>(), p->p1.as<bf>(), n, H[0], W[0], st));
-    RET((conv_launch<C, C, true, bf>(p->p1.p, wf(1), bias_of(p, 1), p->e2.as<bf>(), n, H[1], W[1], de, p->nsm, st)));
-    RET(pool_launch(p->e2.as<bf>(), p->p2.as<bf>(), n, H[1], W[1], st));
-    RET((conv_launch<C, C, true, bf>(p->p2.p, wf(2), bias_of(p, 2), p->e3.as<bf>(), n, H[2], W[2], de, p->nsm, st)));
-    RET(pool_launch(p->e3.as<bf>(), p->p3.as<bf>(), n, H[2], W[2], st));
+    auto pooled = [](Buf &b) {
+        ConvEpi e;
+        e.pool = b.as<bf>();
+        return e;
+    };
+    RET((conv_launch<C, C, true, bf>(p->p1.p, wf(1), bias_of(p, 1), p->e2.as<bf>(), n, H[1], W[1], de, p->nsm, st, pooled(p->p2))));
+    RET((conv_launch<C, C, true, bf>(p->p2.p, wf(2), bias_of(p, 2), p->e3.as<bf>(), n, H[2], W[2], de, p->nsm, st, pooled(p->p3))));
     RET((conv_launch<C, C, true, bf>(p->p3.p, wf(3), bias_of(p, 3), p->bt.as<bf>(), n, H[3], W[3], de, p->nsm, st)));
-    RET(upadd_launch(p->bt.as<bf>(), p->e3.as<bf>(), p->u3.as<bf>(), n, H[2], W[2], st));
-    RET((conv_launch<C, C, true, bf>(p->u3.p, wf(4), bias_of(p, 4), p->d3.as<bf>(), n, H[2], W[2], de, p->nsm, st)));
-    RET(upadd_launch(p->d3.as<bf>(), p->e2.as<bf>(), p->u2.as<bf>(), n, H[1], W[1], st));
-    RET((conv_launch<C, C, true, bf>(p->u2.p, wf(5), bias_of(p, 5), p->d2.as<bf>(), n, H[1], W[1], de, p->nsm, st)));
-    RET(upadd_launch(p->d2.as<bf>(), p->e1.as<bf>(), p->u1.as<bf>(), n, H[0], W[0], st));
-    ConvEpi e6;
+    // the decoder's inputs u = up(coarse) + skip are formed in the convolutions' rings and kept
+    // for the weight gradient only
+    auto sum = [&](const Buf &coarse, Buf &u) {
+        ConvEpi e;
+        e.up = coarse.as<bf>();
+        e.u_out = keep_xn ? u.as<bf>() : nullptr;
+        return e;
+    };
+    RET((conv_launch<C, C, true, bf, true>(p->e3.p, wf(4), bias_of(p, 4), p->d3.as<bf>(), n, H[2], W[2], de, p->nsm, st, sum(p->bt, p->u3))));
+    RET((conv_launch<C, C, true, bf, true>(p->e2.p, wf(5), bias_of(p, 5), p->d2.as<bf>(), n, H[1], W[1], de, p->nsm, st, sum(p->d3, p->u2))));
+    ConvEpi e6 = sum(p->d2, p->u1);
     e6.oscale = p->rms.as<float>();
     e6.nchw = nchw ? 1 : 0;
-    RET((conv_launch<C, G, false, float>(p->u1.p, wf(6), bias_of(p, 6), y, n, H[0], W[0], de, p->nsm, st, e6)));
+    RET((conv_launch<C, G, false, float, true>(p->e1.p, wf(6), bias_of(p, 6), y, n, H[0], W[0], de, p->nsm, st, e6)));
     return cudaSuccess;
 }
 
