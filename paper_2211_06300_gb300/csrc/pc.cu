@@ -170,15 +170,16 @@ __device__ __forceinline__ void store_pixel(float *dst, const float *v) {
 // What bounds it: activation traffic (96 flop/B).  An input row is one TMA box of whole pixels
 // (CIN * 2 bytes) in the swizzle of that width: boxes of one 8-channel chunk each, which the
 // unswizzled layout needs, are CIN/8 times as many 16-byte requests and were the limit, with the
-// barrier per row: the network on 304 images of 121 x 401 took 2.75 ms, 2.07 ms so.  A tap is the row shifted by dx pixels: the slots start on the swizzle's
-// period, so the descriptor's start address moves by whole pixels with base offset 0.
+// barrier per row: the network on 304 images of 121 x 401 took 2.75 ms, 2.07 ms so.  A tap is the
+// row shifted by dx pixels: the slots start on the swizzle's period, so the descriptor's start
+// address moves by whole pixels with base offset 0.
 //
 // Pooling and the decoder's upsample-add are part of the convolutions around them: with epi.pool
 // the epilogue keeps an even row's pixels and writes the 2 x 2 averages with the odd one; with UP
 // the input is epi.up (half the resolution, nearest) + the staged skip row, added in its slot by
 // warps 0 .. 3 one row ahead of the MMAs (`ready` in the place of `full`).  As passes of their own
 // they moved 64 + 16 and 64 + 16 + 64 bytes a pixel and the decoder read 64 again: the same network
-2.07 -> 1.67 ms (first layer with its pooling 428 us, 3.7 TB/s; last one with its sum 568 us).
+// 2.07 -> 1.67 ms (first layer with its pooling 428 us, 3.7 TB/s; last one with its sum 568 us).
 constexpr int RROWS = 6;
 constexpr int NEPI = 4;   // epilogue warps (one TMEM lane quarter each)
 
@@ -474,7 +475,7 @@ __global__ void __launch_bounds__(NTH, CIN == 16 ? 4 : 3) conv3x3_tc_kernel(cons
                         if (epi.pool) {   // y0 is even: the parity of y is the row's
                             static_assert(COUT == 32, "a lane pair averages 16 channels each");
                             if (!(y & 1)) {
-    #pragma unroll
+#pragma unroll
                                 for (int c = 0; c < COUT / 2; ++c) even[c] = pk[c], pk[c] = 0u;
                             }
                             if ((y & 1) || y == ny - 1) {
