@@ -327,9 +327,9 @@ def run_dft3d(args, rank, world, local):
     t_max = shard.max_over_ranks(ms, dist, dev)
     cells_all = shard.sum_over_ranks(cells, dist, dev)
     # the blocked DTFT's bytes per cell update and block length, from the library's profile
-    # entry of the step + fold (FP32: 24 + 16 nf / K bytes)
+    # entry of the step + fold (FP32 in 3D: 20 + 16 nf / K bytes)
     bpc_blk = next(k["bytes_per_cell"] for k in prof if k["name"].endswith("+dft_block"))
-    kblk = int(round(16 * len(freqs) / (bpc_blk - 24)))
+    kblk = int(round(16 * len(freqs) / (bpc_blk - 20)))
     # end to end: the wavelet from pinned host memory in, traces and the FP16 wavefields out
     wav_h = wav.cpu().pin_memory()
     tr_h, U_h = pinned_like(tr), pinned_like(U)
@@ -360,7 +360,7 @@ def run_dft3d(args, rank, world, local):
                              % (4 * w.ncell / 1e6, kblk * 4 * w.ncell / 1e9)},
             # algorithmic bytes per cell update: accumulating every state into the nf complex
             # FP32 accumulators directly costs 16 + 16 nf; the blocked DTFT stashes the states
-            # of a block of K steps and folds them once (16 + 4 stash write + 4 stash read +
+            # of a block of K steps (in 3D they live there) and folds them once (16 + 4 stash read +
             # 16 nf / K), K chosen by the library for the context's memory (from its profile)
             "bytes_per_cell": {"per_step_accumulation": 16 + 16 * len(freqs),
                                "blocked": bpc_blk, "block_steps": kblk},

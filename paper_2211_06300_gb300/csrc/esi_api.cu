@@ -604,10 +604,11 @@ StepArgs<T> base_args(esi_ctx *ctx) {
 }
 
 // One step of either kernel.  In 3D the step kernel samples its input state itself when
-// F_SMP is set (a.tout >= 0), by a gather of the receivers of each block's tile.
+// F_SMP is set (a.tout >= 0), by a gather of the receivers of each block's tile; old: the older
+// state where it is not in a.po.
 template <typename T>
 esi_status step(esi_ctx *ctx, unsigned flags, const StepArgs<T> &a, bool chained = false,
-                int chain = -1) {
+                int chain = -1, const T *old = nullptr) {
     StepArgs<T> b = a;
     cudaStream_t st = ctx->st;
     int ns = ctx->ns;
@@ -617,7 +618,7 @@ esi_status step(esi_ctx *ctx, unsigned flags, const StepArgs<T> &a, bool chained
         ns = ctx->chain_shot(chain + 1) - b.s0;
     }
     if (!state_map(ctx, a.cur, &b.tm) ||
-        (ctx->g.ndim == 3 && (!state_map(ctx, a.po, &b.tm_old, 1) || !state_map(ctx, a.cc, &b.tm_cc, 2))))
+        (ctx->g.ndim == 3 && (!state_map(ctx, old ? old : a.po, &b.tm_old, 1) || !state_map(ctx, a.cc, &b.tm_cc, 2))))
         return ctx->fail(ESI_ERR_CUDA, "cuTensorMapEncodeTiled failed for a state buffer");
     if (ctx->g.ndim == 2) {
         CKL(launch_step2<T>(flags, b, ns, st, chained && ctx->pdl));
@@ -647,9 +648,10 @@ esi_status chains_join(esi_ctx *ctx, esi_status st) {
 
 // one step of every chain
 template <typename T>
-esi_status step_chains(esi_ctx *ctx, unsigned flags, const StepArgs<T> &a, bool chained) {
+esi_status step_chains(esi_ctx *ctx, unsigned flags, const StepArgs<T> &a, bool chained,
+                       const T *old = nullptr) {
     for (int c = 0; c < ctx->chains; ++c) {
-        esi_status st = step<T>(ctx, flags, a, chained, c);
+        esi_status st = step<T>(ctx, flags, a, chained, c, old);
         if (st != ESI_OK) return st;
     }
     return ESI_OK;
@@ -1257,12 +1259,21 @@ esi_status fwd_loop(esi_ctx *ctx, StepArgs<T> a, unsigned flags, T *&cur, T *&po
 
 // Forward modelling with the blocked DTFT: steps [n0, n0 + K) store their new states in the
 // stash, then one launch folds them into the accumulators; the whole run is one graph.
+// In 3D the states live in the stash: a step reads the two slots before its own (across a block's
+// end, the last two of the block just folded) and writes its state once, 16 bytes a cell where a
+// state buffer and the stash took 20.  (2D states stay in L2 and the loops on chip keep theirs.)
 template <typename T>
 esi_status fwd_dft_loop(esi_ctx *ctx, StepArgs<T> a, unsigned flags, T *cur, T *po, T *tr) {
     cudaEvent_t ev = prof_mark(ctx);
     const int nt = ctx->nt;
     auto body = [&](int i0, int i1) -> esi_status {
         T *c = i0 & 1 ? po : cur, *q = i0 & 1 ? cur : po;
+        const bool in_stash = ctx->g.ndim == 3;
+        auto slot = [&](int k) { return a.stash_w + (size_t)k * ctx->ns * ctx->sst; };
+        if (in_stash && i0 > 0) {   // the parts of a graph begin at a block
+            c = slot(ctx->dft_k - 1);
+            q = slot(ctx->dft_k - 2);
+        }
         esi_status e = chains_fork(ctx);
         for (int n0 = i0; n0 < i1 && e == ESI_OK; n0 += ctx->dft_k) {
             const int n1 = std::min(i1, n0 + ctx->dft_k);
@@ -1279,8 +1290,17 @@ esi_status fwd_dft_loop(esi_ctx *ctx, StepArgs<T> a, unsigned flags, T *cur, T *
                 a.tin = n;
                 a.tout = n - 1;
                 a.slot_w = n - n0;
-                e = step_chains<T>(ctx, flags, a, n > i0);
-                std::swap(c, q);
+                if (in_stash) {
+                    StepArgs<T> b = a;
+                    b.po = slot(n - n0);
+                    b.stash_w = nullptr;
+                    e = step_chains<T>(ctx, flags, b, n > i0, q);
+                    q = c;
+                    c = b.po;
+                } else {
+                    e = step_chains<T>(ctx, flags, a, n > i0);
+                    std::swap(c, q);
+                }
             }
             if (e == ESI_OK)
                 e = dft_block_chains<T>(ctx, a.stash_w, n1 - n0, a.nf, a.twid + (size_t)n0 * a.nf * 2, a.dft);
@@ -1297,11 +1317,11 @@ esi_status fwd_dft_loop(esi_ctx *ctx, StepArgs<T> a, unsigned flags, T *cur, T *
         e = body(0, nt);
     }
     if (e != ESI_OK) return e;
-    // the stencil and the stash store per step, plus the block pass: the stash once more
-    // and the accumulators' read and write once per block
+    // the stencil and the stash store per step (in 3D the stash is the state), plus the block
+    // pass: the stash once more and the accumulators' read and write once per block
     const double es = double(sizeof(T));
     prof_close(ctx, ev, step_name(ctx, flags) + "+dft_block",
-               step_bpc(ctx, flags, a.nf) + es + 4.0 * a.nf * es / ctx->dft_k, nt + (nt + ctx->dft_k - 1) / ctx->dft_k,
+               step_bpc(ctx, flags, a.nf) + (ctx->g.ndim == 3 ? 0.0 : es) + 4.0 * a.nf * es / ctx->dft_k, nt + (nt + ctx->dft_k - 1) / ctx->dft_k,
                (long long)nt * ctx->prof_active * ctx->N);
     return ESI_OK;
 }

@@ -68,6 +68,10 @@ __device__ __forceinline__ void tma_load_plane(void *dst, const CUtensorMap *tm,
         : "memory");
 }
 
+__device__ __forceinline__ void prefetch_l1(const void *p) {
+    asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
+}
+
 // Poll the mbarrier phase with an iteration limit; false when the limit ran out.
 __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long *bar, unsigned phase) {
     for (long long i = 0; i < TMA_WAIT_LIMIT; ++i) {
@@ -303,6 +307,16 @@ __global__ void __launch_bounds__(block3<T>(), sizeof(T) == 4 ? ESI_FD3_MINB : 1
             }
             if constexpr ((F & F_AP) != 0) app = ldv3(a.ap_p + fb + (long long)a.nout * a.sst + gi);
         }
+        // The gradient's accumulators and stash are read at the end of the step, at the latency of
+        // L2 or HBM on the march's path, and no registers are left to hold the next plane's: its
+        // lines go to L1 a plane ahead, one thread a line.
+        if constexpr ((F & F_GRD) != 0) {
+            if (rowok && lx * sizeof(T) % 128 == 0 && i + 1 < nsteps) {
+                const long long gn = (long long)s * a.sst + gi + plane;
+                prefetch_l1(a.grad + gn);
+                prefetch_l1(a.stash_r + (long long)a.slot_r * a.ns * a.sst + gn);
+            }
+        }
         // plane z (sequence index i + 4) has landed: the queue fill waited for it when
         // i + 4 <= 8, else the refill at the end of step i - 5; its slot is not reused
         // before this warp releases it at the end of this step
@@ -485,8 +499,8 @@ __global__ void __launch_bounds__(block3<T>(), sizeof(T) == 4 ? ESI_FD3_MINB : 1
                         if (gx0 + k < a.nx) o[k] = nw.v[k];
                 }
             }
-            if constexpr ((F & F_DFT) != 0)   // the DTFT's block stash (slot n - n0)
-                stv3(a.stash_w + ((long long)a.slot_w * a.ns + s) * a.sst + gi, nw);
+            if constexpr ((F & F_DFT) != 0)   // the DTFT's block stash, unless po is its slot
+                if (a.stash_w) stv3(a.stash_w + ((long long)a.slot_w * a.ns + s) * a.sst + gi, nw);
         }
     };
     // after step O of the group that starts at plane i: the next plane into the queue (once
