@@ -1293,8 +1293,7 @@ esi_status fwd_dft_loop(esi_ctx *ctx, StepArgs<T> a, unsigned flags, T *cur, T *
                 if (in_stash) {
                     StepArgs<T> b = a;
                     b.po = slot(n - n0);
-                    b.stash_w = nullptr;
-                    e = step_chains<T>(ctx, flags, b, n > i0, q);
+                    e = step_chains<T>(ctx, flags & ~F_DFT, b, n > i0, q);
                     q = c;
                     c = b.po;
                 } else {

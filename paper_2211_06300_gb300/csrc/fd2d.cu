@@ -19,7 +19,10 @@
 //   epilogue : output of the new state, CG product Ap = new + beta B^2 p with the <p, Ap>
 //              block partial, gradient stash / correlation, saddle-point correlation,
 //              on-the-fly DTFT accumulation.
+#include <type_traits>
+
 #include "esi_internal.h"
+#include "pairs.h"
 
 namespace esi {
 namespace {
@@ -77,6 +80,11 @@ __device__ __forceinline__ void stv(T *p, const Vec<T> &v) {
 __device__ __forceinline__ void prefetch_l1(const void *p) {
     asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
 }
+
+// Cell pairs halve the Laplacian's issue slots, except in the two halves of the CG product, whose 64
+// registers they overflow (solve of 16 shots of 801 x 241: 78.1 ms with, 77.3 without).
+template <typename T, unsigned F>
+using StepPk = std::conditional_t<sizeof(T) == 4 && (F & (F_AP | F_CGP)) != 0, PkCell, Pk<T>>;
 
 template <typename T, unsigned F>
 __global__ void __launch_bounds__(NT2, MINB2) fd2_step_kernel(const __grid_constant__ StepArgs<T> a) {
@@ -243,27 +251,48 @@ __global__ void __launch_bounds__(NT2, MINB2) fd2_step_kernel(const __grid_const
             const int gz = z0 + lz;
             if (gz >= a.nz) break;
             const int sz = lz + HALO;
-            // x neighbours: shared row segment [lx, lx + VEC + 8)
+            // x neighbours: shared row segment [lx, lx + VEC + 8), in pairs of cells
+            using P = StepPk<T, F>;
+            using S16 = Seg<T, P>;
+            constexpr int HP = HALO / P::n;   // pairs of a halo
+            typename P::t wp[2 * HP + S16::n];
             T w[VEC + 2 * HALO];
 #pragma unroll
             for (int c = 0; c < (VEC + 2 * HALO) / VEC; ++c) {
-                const Vec<T> t = ldv(&tl[sz][lx + c * VEC]);
+                const S16 t = ldp<T, P>(&tl[sz][lx + c * VEC]);
 #pragma unroll
-                for (int i = 0; i < VEC; ++i) w[c * VEC + i] = t.v[i];
+                for (int j = 0; j < S16::n; ++j) {
+                    wp[S16::n * c + j] = t.v[j];
+                    P::unpack(t.v[j], w + (S16::n * c + j) * P::n);
+                }
             }
             // Laplacian sum: 2 w0 u + sum_k w_k (4 neighbours at distance k)
-            T L[VEC];
-#pragma unroll
-            for (int i = 0; i < VEC; ++i) L[i] = T(2.0 * W0) * w[i + HALO];
+            typename P::t Lp[S16::n];
             constexpr double WZ[5] = {0.0, W1, W2, W3, W4};
 #pragma unroll
             for (int k = 1; k <= HALO; ++k) {
-                const Vec<T> up = ldv(&tl[sz - k][lx + HALO]);
-                const Vec<T> dn = ldv(&tl[sz + k][lx + HALO]);
+                const S16 up = ldp<T, P>(&tl[sz - k][lx + HALO]);
+                const S16 dn = ldp<T, P>(&tl[sz + k][lx + HALO]);
 #pragma unroll
-                for (int i = 0; i < VEC; ++i)
-                    L[i] += T(WZ[k]) * ((w[i + HALO - k] + w[i + HALO + k]) + (up.v[i] + dn.v[i]));
+                for (int j = 0; j < S16::n; ++j) {
+                    typename P::t x2;
+                    if (k % P::n == 0) {
+                        x2 = P::add(wp[HP + j - k / P::n], wp[HP + j + k / P::n]);
+                    } else {   // neighbours that are no whole pairs
+                        T t[P::n];
+#pragma unroll
+                        for (int i = 0; i < P::n; ++i)
+                            t[i] = w[j * P::n + i + HALO - k] + w[j * P::n + i + HALO + k];
+                        x2 = P::pack(t);
+                    }
+                    const typename P::t sum = P::add(x2, P::add(up.v[j], dn.v[j]));
+                    Lp[j] = k == 1 ? P::fma(P::dup(T(2.0 * W0)), wp[HP + j], P::mul(P::dup(T(W1)), sum))
+                                   : P::fma(P::dup(T(WZ[k])), sum, Lp[j]);
+                }
             }
+            T L[VEC];
+#pragma unroll
+            for (int j = 0; j < S16::n; ++j) P::unpack(Lp[j], L + j * P::n);
             const long long gi = (long long)gz * a.px + gx0;
             const Vec<T> old = p_old[pz];
             const Vec<T> cc = p_cc[pz];

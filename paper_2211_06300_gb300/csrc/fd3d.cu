@@ -20,6 +20,7 @@
 #include <type_traits>
 
 #include "esi_internal.h"
+#include "pairs.h"
 
 namespace esi {
 
@@ -115,10 +116,6 @@ constexpr int ring_bytes() {
 #define ESI_FD3_UNROLL 4
 #endif
 static_assert(ESI_FD3_UNROLL >= 1 && ESI_FD3_UNROLL <= 4, "unroll 1..4");
-// the centre cells of a row come from the register queue (else from shared memory)
-#ifndef ESI_FD3_WQ
-#define ESI_FD3_WQ 1
-#endif
 
 template <typename T, unsigned F>
 __global__ void __launch_bounds__(block3<T>(), sizeof(T) == 4 ? ESI_FD3_MINB : 1) fd3_step_kernel(const __grid_constant__ StepArgs<T> a,
@@ -242,13 +239,13 @@ __global__ void __launch_bounds__(block3<T>(), sizeof(T) == 4 ? ESI_FD3_MINB : 1
     };
     bool late = false;
     constexpr int UN = ESI_FD3_UNROLL;
-    T q[2 * HALO + UN][VEC];   // u(z - 4 .. z + 4) of the row segment, + UN - 1 planes ahead
+    using P = Pk<T>;
+    typename P::t q[2 * HALO + UN][2];   // u(z - 4 .. z + 4) of the row segment, + UN - 1 planes ahead
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
         late |= !ready(k);
-        const Vec3<T> c = ldv3(&ring[k % RING3].u[ry + HALO][lx + HALO]);
-#pragma unroll
-        for (int i = 0; i < VEC; ++i) q[k][i] = c.v[i];
+        const Seg<T> c = ldp(&ring[k % RING3].u[ry + HALO][lx + HALO]);
+        q[k][0] = c.v[0], q[k][1] = c.v[1];
         // planes zb - 4 .. zb - 1 serve only their centres: free their slots at once (the
         // ring holds fewer than the 9 planes of the queue)
         if (k < HALO) release(k);
@@ -325,6 +322,7 @@ __global__ void __launch_bounds__(block3<T>(), sizeof(T) == 4 ? ESI_FD3_MINB : 1
         // warp scans them 32 at a time, each lane sums the entries of the warp's rows it
         // holds and leaves the sum in the owner's slot of the warp's scratch
         bool has_inj = false;
+        (void)has_inj;
         if constexpr ((F & F_PT) != 0) {
             if (ip < ie && a.inj.cell[ip] / (TX3 * TY3) == z) {   // uniform in the warp
                 has_inj = true;
@@ -361,45 +359,53 @@ __global__ void __launch_bounds__(block3<T>(), sizeof(T) == 4 ? ESI_FD3_MINB : 1
         }
         if (rowok) {
             const int sy = ry + HALO;
-            // x neighbours: the shared row segment [lx, lx + VEC + 8); its centre part is the
-            // plane's own cells, already in the register queue
-            T w[VEC + 2 * HALO];
-#if ESI_FD3_WQ
+            // x neighbours: the shared row segment [lx, lx + VEC + 8) in pairs; its centre part is
+            // the plane's own cells, already in the register queue
+            constexpr int HP = HALO / P::n;   // pairs of a halo
+            typename P::t w[2 * HP + 2];
 #pragma unroll
-            for (int c = 0; c < HALO / VEC; ++c) {
-                const Vec3<T> tl = ldv3(&sl.u[sy][lx + c * VEC]);
-                const Vec3<T> tr = ldv3(&sl.u[sy][lx + HALO + VEC + c * VEC]);
+            for (int c = 0; c < HP / 2; ++c) {
+                const Seg<T> tl = ldp(&sl.u[sy][lx + c * VEC]);
+                const Seg<T> tr = ldp(&sl.u[sy][lx + HALO + VEC + c * VEC]);
 #pragma unroll
-                for (int k = 0; k < VEC; ++k) {
-                    w[c * VEC + k] = tl.v[k];
-                    w[HALO + VEC + c * VEC + k] = tr.v[k];
+                for (int j = 0; j < 2; ++j) {
+                    w[2 * c + j] = tl.v[j];
+                    w[HP + 2 + 2 * c + j] = tr.v[j];
                 }
             }
 #pragma unroll
-            for (int k = 0; k < VEC; ++k) w[HALO + k] = q[O + HALO][k];
-#else
-#pragma unroll
-            for (int c = 0; c < (VEC + 2 * HALO) / VEC; ++c) {
-                const Vec3<T> t = ldv3(&sl.u[sy][lx + c * VEC]);
-#pragma unroll
-                for (int k = 0; k < VEC; ++k) w[c * VEC + k] = t.v[k];
-            }
-#endif
+            for (int j = 0; j < 2; ++j) w[HP + j] = q[O + HALO][j];
             // Laplacian sum: 3 w0 u + sum_k w_k (6 neighbours at distance k)
-            T L[VEC];
-#pragma unroll
-            for (int k = 0; k < VEC; ++k) L[k] = T(3.0 * W0) * q[O + HALO][k];
+            typename P::t L[2];
 #pragma unroll
             for (int d = 1; d <= HALO; ++d) {
-                const Vec3<T> up = ldv3(&sl.u[sy - d][lx + HALO]);
-                const Vec3<T> dn = ldv3(&sl.u[sy + d][lx + HALO]);
+                const Seg<T> up = ldp(&sl.u[sy - d][lx + HALO]);
+                const Seg<T> dn = ldp(&sl.u[sy + d][lx + HALO]);
+                // the neighbours along x: whole pairs at distances that are pairs, else by cell
+                typename P::t xs2[2];
+                if (d % P::n == 0) {
 #pragma unroll
-                for (int k = 0; k < VEC; ++k)
-                    L[k] += T(WK[d]) * (((w[k + HALO - d] + w[k + HALO + d]) + (up.v[k] + dn.v[k])) +
-                                        (q[O + HALO - d][k] + q[O + HALO + d][k]));
+                    for (int j = 0; j < 2; ++j) xs2[j] = P::add(w[HP + j - d / P::n], w[HP + j + d / P::n]);
+                } else {
+                    T e[2 * HALO + VEC];
+#pragma unroll
+                    for (int j = 0; j < 2 * HP + 2; ++j) P::unpack(w[j], e + j * P::n);
+                    T t[VEC];
+#pragma unroll
+                    for (int k = 0; k < VEC; ++k) t[k] = e[k + HALO - d] + e[k + HALO + d];
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) xs2[j] = P::pack(t + j * P::n);
+                }
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const typename P::t sum = P::add(P::add(xs2[j], P::add(up.v[j], dn.v[j])),
+                                                     P::add(q[O + HALO - d][j], q[O + HALO + d][j]));
+                    L[j] = d == 1 ? P::fma(P::dup(T(3.0 * W0)), q[O + HALO][j], P::mul(P::dup(T(W1)), sum))
+                                  : P::fma(P::dup(T(WK[d])), sum, L[j]);
+                }
             }
-            const Vec3<T> old = ldv3(&sl.old[ry][lx]);
-            const Vec3<T> cz = ldv3(&sl.c[ry][lx]);
+            const Seg<T> old = ldp(&sl.old[ry][lx]);
+            const Seg<T> cz = ldp(&sl.c[ry][lx]);
             T src[VEC], S[VEC];
 #pragma unroll
             for (int k = 0; k < VEC; ++k) src[k] = T(0);
@@ -424,28 +430,41 @@ __global__ void __launch_bounds__(block3<T>(), sizeof(T) == 4 ? ESI_FD3_MINB : 1
                 for (int k = 0; k < VEC; ++k) src[k] += pn.v[k];
             }
 #pragma unroll
-            for (int k = 0; k < VEC; ++k) S[k] = L[k] + a.dx2 * src[k];
+            for (int j = 0; j < 2; ++j) {
+                if constexpr ((F & (F_EXT | F_CGP)) != 0)
+                    L[j] = P::fma(P::dup(a.dx2), P::pack(src + j * P::n), L[j]);
+            }
             if constexpr ((F & F_PT) != 0) {
                 if (has_inj) {   // this plane's point sums, gathered by the warp
+                    const Seg<T> pt = ldp(&scr[lane * VEC]);
 #pragma unroll
-                    for (int k = 0; k < VEC; ++k) S[k] += scr[lane * VEC + k];
+                    for (int j = 0; j < 2; ++j) L[j] = P::add(L[j], pt.v[j]);
                 }
             }
+#pragma unroll
+            for (int j = 0; j < 2; ++j) P::unpack(L[j], S + j * P::n);
             Vec3<T> nw;
             if (xy_sponge || kzz != T(0)) {
+                T un[VEC], on[VEC], cn[VEC];
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    P::unpack(q[O + HALO][j], un + j * P::n);
+                    P::unpack(old.v[j], on + j * P::n);
+                    P::unpack(cz.v[j], cn + j * P::n);
+                }
 #pragma unroll
                 for (int k = 0; k < VEC; ++k) {
                     const T kap = kzz + kxy[k];
                     const T al = T(1) / (T(1) + kap);
                     const T ga = (T(1) - kap) * al;
-                    const T u = q[O + HALO][k];
-                    nw.v[k] = u + ga * (u - old.v[k]) + al * cz.v[k] * S[k];
+                    const T u = un[k];
+                    nw.v[k] = u + ga * (u - on[k]) + al * cn[k] * S[k];
                 }
             } else {   // interior: alpha = gamma = 1
 #pragma unroll
-                for (int k = 0; k < VEC; ++k) {
-                    const T u = q[O + HALO][k];
-                    nw.v[k] = u + (u - old.v[k]) + cz.v[k] * S[k];
+                for (int j = 0; j < 2; ++j) {
+                    const typename P::t u = q[O + HALO][j];
+                    P::unpack(P::fma(cz.v[j], L[j], P::add(u, P::sub(u, old.v[j]))), nw.v + j * P::n);
                 }
             }
 #pragma unroll
@@ -499,8 +518,8 @@ __global__ void __launch_bounds__(block3<T>(), sizeof(T) == 4 ? ESI_FD3_MINB : 1
                         if (gx0 + k < a.nx) o[k] = nw.v[k];
                 }
             }
-            if constexpr ((F & F_DFT) != 0)   // the DTFT's block stash, unless po is its slot
-                if (a.stash_w) stv3(a.stash_w + ((long long)a.slot_w * a.ns + s) * a.sst + gi, nw);
+            if constexpr ((F & F_DFT) != 0)   // the DTFT's block stash (slot n - n0)
+                stv3(a.stash_w + ((long long)a.slot_w * a.ns + s) * a.sst + gi, nw);
         }
     };
     // after step O of the group that starts at plane i: the next plane into the queue (once
@@ -510,9 +529,8 @@ __global__ void __launch_bounds__(block3<T>(), sizeof(T) == 4 ? ESI_FD3_MINB : 1
         if constexpr (O + 1 < UN) {
             if (i + O + 1 < nsteps) {   // plane z + 5 of the next step into entry O + 9
                 late |= !ready(i + O + 2 * HALO + 1);
-                const Vec3<T> c = ldv3(&ring[(i + O + 2 * HALO + 1) % RING3].u[ry + HALO][lx + HALO]);
-#pragma unroll
-                for (int e = 0; e < VEC; ++e) q[O + 2 * HALO + 1][e] = c.v[e];
+                const Seg<T> c = ldp(&ring[(i + O + 2 * HALO + 1) % RING3].u[ry + HALO][lx + HALO]);
+                q[O + 2 * HALO + 1][0] = c.v[0], q[O + 2 * HALO + 1][1] = c.v[1];
             }
         } else {
             if (i + UN < nsteps) {
@@ -520,10 +538,9 @@ __global__ void __launch_bounds__(block3<T>(), sizeof(T) == 4 ? ESI_FD3_MINB : 1
 #pragma unroll
                 for (int k = 0; k < 2 * HALO; ++k)
 #pragma unroll
-                    for (int e = 0; e < VEC; ++e) q[k][e] = q[k + UN][e];
-                const Vec3<T> c = ldv3(&ring[(i + UN + 2 * HALO) % RING3].u[ry + HALO][lx + HALO]);
-#pragma unroll
-                for (int e = 0; e < VEC; ++e) q[2 * HALO][e] = c.v[e];
+                    for (int e = 0; e < 2; ++e) q[k][e] = q[k + UN][e];
+                const Seg<T> c = ldp(&ring[(i + UN + 2 * HALO) % RING3].u[ry + HALO][lx + HALO]);
+                q[2 * HALO][0] = c.v[0], q[2 * HALO][1] = c.v[1];
             }
         }
         release(i + O + HALO);   // plane z: its neighbours and centre were last read in this step
