@@ -306,7 +306,8 @@ __global__ void __launch_bounds__(block3<T>(), sizeof(T) == 4 ? ESI_FD3_MINB : 1
         }
         // The gradient's accumulators and stash are read at the end of the step, at the latency of
         // L2 or HBM on the march's path, and no registers are left to hold the next plane's: its
-        // lines go to L1 a plane ahead, one thread a line.
+        // lines go to L1 a plane ahead, one thread a line (gradient of two shots of 150 x 131 x
+        // 187: 22.76 -> 21.75 ms).
         if constexpr ((F & F_GRD) != 0) {
             if (rowok && lx * sizeof(T) % 128 == 0 && i + 1 < nsteps) {
                 const long long gn = (long long)s * a.sst + gi + plane;
