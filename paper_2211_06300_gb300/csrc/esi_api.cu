@@ -2461,7 +2461,9 @@ esi_status fdcg_impl(esi_ctx *ctx, double lambda, double tol, int max_iter, cons
                     a.n = n - n0;   // the stash slot
                     a.tin = n;
                     a.tout = n - 1;
-                    st = step_chains<T>(ctx, F_CGP | F_SMP, a, n > i0);
+                    // not a dependent launch behind the synthesis: the step reads its sources
+                    // before it waits for the launch in front of it
+                    st = step_chains<T>(ctx, F_CGP | F_SMP, a, n > n0);
                     std::swap(c, q);
                 }
             }
