@@ -851,6 +851,7 @@ struct LoopInjHost {
             for (int t = 0; t < tiles; ++t) {
                 int blk = -1, cell = -1, np = 0;
                 const size_t i0 = inj.size();
+                std::vector<std::pair<int, int>> cells;   // place, first contribution
                 for (; k < nodes.size() && nodes[k].tile == t; ++k) {
                     const Node &n = nodes[k];
                     if (n.blk != blk) {
@@ -858,8 +859,14 @@ struct LoopInjHost {
                         blk = n.blk, cell = -1;
                         ++np;
                     }
-                    inj.push_back({n.con.off0, n.con.tstride, n.cell == cell ? -1 : (np - 1) * 16 + n.cell, T(n.con.w)});
+                    if (n.cell != cell) cells.push_back({(np - 1) * 16 + n.cell, (int)(inj.size() - i0)});
                     cell = n.cell;
+                    inj.push_back({n.con.off0, n.con.tstride, LOOP_NONE, 0, T(n.con.w), T(0)});
+                }
+                // (numbers beyond 16 bits come with lists beyond the shared memory)
+                for (size_t i = 0; i < cells.size(); ++i) {
+                    inj[i0 + i].pos = (unsigned short)cells[i].first;
+                    inj[i0 + i].first = (unsigned short)cells[i].second;
                 }
                 ptr.push_back((int)inj.size());
                 patch_ptr.push_back((int)patch_blk.size());

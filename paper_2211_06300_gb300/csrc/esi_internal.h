@@ -195,13 +195,17 @@ __host__ __device__ inline int loop_part(int i, int parts, int n) {
     return (int)((long long)i * n / parts);
 }
 
-// one contribution to a point-source cell: value w * trace[off + t * stride]; pos = the cell's
-// place in the tile's patches (16 values per block), or -1 when it adds to the entry before it
+// Entry i of a tile's point-source list: its i-th contribution, w * trace[off + t * stride] (v: the
+// tile's copy of the trace value), and its i-th cell that has any: the cell's place in the tile's
+// patches (16 values per block; LOOP_NONE past the last cell) and its first contribution.  Both
+// run in the same order, so a cell's contributions end where the next cell's begin.
+constexpr unsigned short LOOP_NONE = 0xffff;
 template <typename T>
 struct LoopInj {
     long long off;
-    int stride, pos;
-    T w;
+    int stride;
+    unsigned short pos, first;
+    T w, v;
 };
 // one receiver: four points of the tile's shared-memory array, and its trace
 template <typename T>

@@ -41,6 +41,7 @@ constexpr double W0 = -205.0 / 72.0, W1 = 8.0 / 5.0, W2 = -1.0 / 5.0, W3 = 8.0 /
 // polls of a packet before a wait gives up (about 0.6 us each: seconds)
 constexpr int POLL_LIMIT = 1 << 22;
 constexpr int SMP_T = 32;     // of the communication threads: those that sample the receivers
+constexpr int INJ_U = 4;      // trace values a thread has in flight for the point sources
 constexpr int PF_AHEAD = 2;   // steps by which the streams' L2 prefetch runs ahead
 
 // The cells of one thread along x: four FP32 as two packed pairs (f32x2 instructions halve the
@@ -293,19 +294,46 @@ __global__ void __launch_bounds__(LOOP_THREADS, 1)
             for (int i = tid; i < np; i += nthr) map[g.patch_blk[pb + i]] = (unsigned short)(i + 1);
         }
         __syncthreads();
-        // the sum of a node's contributions (usually one) at trace time t, by its first entry
-        auto inject = [&](int c, int t) -> T {
-            T sum = T(0);
-            do {
-                const LoopInj<T> e = inj[c];
-                sum += e.w * a.inj_trace[e.off + (long long)t * e.stride];
-                ++c;
-            } while (c < nci && inj[c].pos < 0);
-            return sum;
+        // The point-source cells at trace time t into the patch set p, by the `n` threads that call
+        // this as me = 0 .. n - 1.  A cell's contributions (usually one) are added in list order.
+        // Loads of a thread's entries go out INJ_U at a time: an entry is the latency of L2 or HBM,
+        // and a tile can hold thousands.  Where a cell has several, all threads load, and a thread
+        // per cell adds them up from shared memory.  (2000 receivers on a line, back-propagation, us
+        // per step, with one load at a time by the cell's thread and so: one shot of 101 x 101 33 and
+        // 3.0, 20 shots of 97 x 130 68 and 4.9; the per-step kernel 7.7 and 8.1.)
+        bool several = false;
+        auto inject = [&](T *p, int t, int me, int n, auto &&sync) {
+            for (int c0 = me; c0 < nci; c0 += INJ_U * n) {
+                T v[INJ_U];
+#pragma unroll
+                for (int u = 0; u < INJ_U; ++u) {
+                    const int c = c0 + u * n;
+                    v[u] = c < nci ? a.inj_trace[inj[c].off + (long long)t * inj[c].stride] : T(0);
+                }
+#pragma unroll
+                for (int u = 0; u < INJ_U; ++u) {
+                    const int c = c0 + u * n;
+                    if (c >= nci) break;
+                    T sum = T(0);
+                    sum += inj[c].w * v[u];
+                    if (several) inj[c].v = v[u];
+                    else p[inj[c].pos] = sum;
+                }
+            }
+            if (!several) return;
+            sync();
+            for (int i = me; i < nci && inj[i].pos != LOOP_NONE; i += n) {
+                const int end = i + 1 < nci && inj[i + 1].pos != LOOP_NONE ? inj[i + 1].first : nci;
+                T sum = T(0);
+#pragma unroll 4
+                for (int c = inj[i].first; c < end; ++c) sum += inj[c].w * inj[c].v;
+                p[inj[i].pos] = sum;
+            }
         };
         if constexpr ((F & F_PT) != 0) {
-            for (int c = tid; c < nci; c += nthr)
-                if (inj[c].pos >= 0) patch[inj[c].pos] = inject(c, a.tin);
+            if (tid == 0 && nci > 0) several = inj[nci - 1].pos == LOOP_NONE;
+            several = __syncthreads_or(several);
+            inject(patch, a.tin, tid, nthr, [] { __syncthreads(); });
             __syncthreads();
         }
 
@@ -557,9 +585,8 @@ __global__ void __launch_bounds__(LOOP_THREADS, 1)
                     if (k + 1 < g.steps) {
                         // the next step's point sources, into the other patch set
                         if constexpr ((F & F_PT) != 0) {
-                            T *pn = patch + ((k + 1) & 1) * 16 * np;
-                            for (int c = ct; c < nci; c += nxt)
-                                if (inj[c].pos >= 0) pn[inj[c].pos] = inject(c, a.tin + dk + g.dn);
+                            inject(patch + ((k + 1) & 1) * 16 * np, a.tin + dk + g.dn, ct, nxt,
+                                   [&] { asm volatile("barrier.sync 1, %0;" ::"r"(nxt) : "memory"); });
                         }
                         // the halo of the new state: entries [above][below][left][right]
                         const ulonglong2 *box = ((k & 1) ? in1 : in0) + (long long)me * g.istride;
