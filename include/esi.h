@@ -28,10 +28,16 @@
  *  Streams   : all work is enqueued on the stream given to esi_create (or
  *              esi_set_stream).  Calls return after enqueueing, except where stated
  *              (esi_cg_solve, esi_gradient's misfit, esi_dft_extract's scales), which
- *              synchronise the stream to read a few scalars back.
+ *              synchronise the stream to read a few scalars back.  A time loop in 2D may run
+ *              as cooperative launches of many steps each, which hold one block per SM, or
+ *              half of its shots on a second, internal stream, which the context's stream
+ *              waits for.
  *  Errors    : every call returns an esi_status; nothing is thrown across the ABI.  On
- *              failure esi_last_error(ctx) gives a message.  A context whose call failed
- *              with ESI_ERR_CUDA should be destroyed.
+ *              failure esi_last_error(ctx) gives a message.  Every wait inside a kernel is
+ *              bounded; one that runs out leaves results unfinished.  A call that
+ *              synchronises then returns ESI_ERR_TIMEOUT; after a call that only enqueues,
+ *              esi_synchronize and every later call on the context (or network) do.  A context
+ *              whose call failed with ESI_ERR_CUDA or ESI_ERR_TIMEOUT should be destroyed.
  */
 #ifndef ESI_H
 #define ESI_H
@@ -103,6 +109,12 @@ ESI_API void esi_destroy(esi_ctx *ctx);
 /* Replace the context's stream (cudaStream_t). */
 ESI_API esi_status esi_set_stream(esi_ctx *ctx, void *stream);
 
+/*
+ * esi_synchronize -- wait for the work queued on the context's stream and report what became of
+ * it: ESI_OK, ESI_ERR_CUDA, or ESI_ERR_TIMEOUT when a device wait of any call so far ran out.
+ */
+ESI_API esi_status esi_synchronize(esi_ctx *ctx);
+
 /* Replace the velocity model (same grid, same sponge reference); device pointer.  Shot
  * groups (esi_set_shot_groups) follow it. */
 ESI_API esi_status esi_set_velocity(esi_ctx *ctx, const void *velocity_dev);
@@ -160,9 +172,11 @@ ESI_API esi_status esi_forward(esi_ctx *ctx, const void *wavelet_dev, const void
  *               at the start of every call, so results do not depend on earlier calls,
  *               but calls whose work overlaps on the GPU (other streams, other threads,
  *               other contexts on the same device) race on it: serialise them.
- *   Launches  : the step kernels of esi_forward, issued one by one (no CUDA graph, since
- *               instantiating one may take device memory), every step after the first a
- *               programmatic dependent launch; recorded by esi_get_profile like esi_forward.
+ *   Launches  : one step kernel a step (where esi_forward may run many steps in one launch, or
+ *               the shots in two chains of launches: the same operations per cell, the same
+ *               results), issued one by one (no CUDA graph, since instantiating one may take
+ *               device memory), every step after the first a programmatic dependent launch;
+ *               recorded by esi_get_profile like esi_forward.
  *   Arguments : as esi_forward; traces_dev must not be NULL.
  */
 ESI_API esi_status esi_forward_noalloc(esi_ctx *ctx, const void *wavelet_dev,

@@ -97,6 +97,32 @@ struct LoopPlan {
 
 }  // namespace
 
+namespace esi {
+cudaError_t ErrWord::make() {
+    std::lock_guard<std::recursive_mutex> lk(g_dev_mu);
+    cudaError_t e = cudaHostAlloc((void **)&h, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable);
+    if (e != cudaSuccess) return e;
+    *h = 0;
+    return cudaHostGetDevicePointer((void **)&d, h, 0);
+}
+ErrWord::~ErrWord() {
+    if (!h) return;
+    std::lock_guard<std::recursive_mutex> lk(g_dev_mu);
+    cudaFreeHost(h);
+}
+const char *ErrWord::text() const {
+    switch (h ? *(const volatile int *)h : 0) {
+        case 0: return nullptr;
+        case DEV_ERR_LOOP_TIMEOUT:
+            return "a device wait ran out: a tile of an on-chip time loop did not get its neighbours' "
+                   "rims (results since then are not valid)";
+        default:
+            return "a device wait ran out: a TMA tile or tensor-core accumulator did not arrive within "
+                   "its iteration limit (results since then are not valid)";
+    }
+}
+}  // namespace esi
+
 struct esi_ctx {
     esi_grid g{};
     int ns = 0, nt = 0;
@@ -114,7 +140,7 @@ struct esi_ctx {
     DBuf ac;                       // alpha c (2D: the on-chip loops)
     // sponge rows [0, spz[0]) and [spz[1], nz) and columns likewise, where kappa is not zero
     int spz[2] = {0, 0}, spx[2] = {0, 0};
-    DBuf dev_err;                  // sticky device error word (int)
+    ErrWord dev_err;               // a bounded device wait ran out
     struct TMap {
         const void *base;
         int kind;
@@ -194,6 +220,7 @@ struct esi_ctx {
     cudaEvent_t chain_ev[2] = {nullptr, nullptr};   // fork, join
     int chain_shot(int c) const { return c * ns / chains; }   // its first shot (c = chains: the end)
     cudaStream_t chain_stream(int c) const { return c ? chain_st : st; }
+    int loop_polls = LOOP_POLLS;   // of a rim packet of the on-chip loops, before a wait gives up
     bool use_graphs = true;
     bool pdl = true;               // loop steps after the first start as dependent launches
     unsigned long long graph_clock = 0;
@@ -599,7 +626,7 @@ StepArgs<T> base_args(esi_ctx *ctx) {
     a.src_pos = ctx->src_pos.as<double>();
     a.ns = ctx->ns;
     a.tout = -1;
-    a.dev_err = ctx->dev_err.as<int>();
+    a.dev_err = ctx->dev_err.d;
     return a;
 }
 
@@ -1066,15 +1093,22 @@ esi_status ensure_states(esi_ctx *ctx, bool adj) {
     return ESI_OK;
 }
 
-// Reads the sticky device error word (after a synchronisation point of the call).
+// What the sticky error word says so far.
+esi_status dev_err_status(esi_ctx *ctx) {
+    const char *t = ctx->dev_err.text();
+    return t ? ctx->fail(ESI_ERR_TIMEOUT, t) : ESI_OK;
+}
+
+// The same after the work queued on the context stream.
 esi_status check_dev_err(esi_ctx *ctx) {
-    int h = 0;
-    CK(cudaMemcpyAsync(&h, ctx->dev_err.p, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
     CK(cudaStreamSynchronize(ctx->st));
-    if (h == DEV_ERR_TMA_TIMEOUT)
-        return ctx->fail(ESI_ERR_TIMEOUT, "a TMA tile wait ran out of its iteration limit");
-    if (h) return ctx->fail(ESI_ERR_TIMEOUT, "device error word " + std::to_string(h));
-    return ESI_OK;
+    return dev_err_status(ctx);
+}
+
+// Start of a call: no message yet, and no wait of an earlier call has run out.
+esi_status begin_call(esi_ctx *ctx) {
+    ctx->err.clear();
+    return dev_err_status(ctx);
 }
 
 // ------------------------------------------------------------------ loop graphs
@@ -1193,6 +1227,7 @@ esi_status loop_run(esi_ctx *ctx, unsigned flags, StepArgs<T> a, T *cur, T *po, 
     g.qx = (ctx->g.nx + 3) / 4, g.gr = (ctx->g.nz + 3) / 4;
     g.steps = steps, g.dn = dn, g.nt = ctx->nt;
     g.nc = lp.nc, g.nm = LOOP_COMM;
+    g.polls = ctx->loop_polls;
     g.lanes = lp.lanes;
     g.nbz0 = ctx->spz[0], g.nbz1 = ctx->spz[1], g.nbx0 = ctx->spx[0], g.nbx1 = ctx->spx[1];
     g.ac = ctx->ac.as<T>();
@@ -1666,6 +1701,7 @@ esi_status gradient_impl(esi_ctx *ctx, const void *wavelet, const void *ext, con
             double J = h[0];
             for (int s = 0; s < ns; ++s) J += h[1 + s];
             *misfit = J;
+            if ((e = dev_err_status(ctx)) != ESI_OK) return e;
         }
     } else {
         if (!wavelet && !ext) return ctx->fail(ESI_ERR_ARG, "no source given");
@@ -1779,7 +1815,7 @@ esi_status dft_impl(esi_ctx *ctx, const void *wavelet, const void *ext, const do
     if (half) {
         CK(cudaMemcpyAsync(scales, ctx->ckpt_scale.p, sizeof(float) * ctx->ns * nf,
                            cudaMemcpyDeviceToHost, ctx->st));
-        CK(cudaStreamSynchronize(ctx->st));
+        return check_dev_err(ctx);
     }
     return ESI_OK;
 }
@@ -2818,8 +2854,7 @@ esi_status invert_impl(esi_ctx *ctx, const esi_invert_opts *o, const void *wavel
 
 template <typename T>
 esi_status create_impl(esi_ctx *ctx, const void *vel) {
-    CK(ctx->dev_err.ensure(sizeof(int)));
-    CK(cudaMemsetAsync(ctx->dev_err.p, 0, sizeof(int), ctx->st));
+    CK(ctx->dev_err.make());
     esi_status e = setup_model<T>(ctx, vel, true);
     if (e != ESI_OK) return e;
     e = setup_geometry<T>(ctx);
@@ -3090,6 +3125,7 @@ esi_status create_ctx(esi_ctx **out, const esi_grid *grid, const esi_geometry *g
     }
     if (const char *ev = std::getenv("ESI_NO_GRAPHS")) ctx->use_graphs = ev[0] == '0';
     if (const char *ev = std::getenv("ESI_PDL")) ctx->pdl = ev[0] != '0';
+    if (const char *ev = std::getenv("ESI_LOOP_POLLS")) ctx->loop_polls = std::max(0, std::atoi(ev));
     esi_ctx *c = ctx.get();
     {
         esi_ctx *ctx = c;  // for CK
@@ -3123,6 +3159,16 @@ ESI_API esi_status esi_set_stream(esi_ctx *ctx, void *stream) {
     return ESI_OK;
 }
 
+
+ESI_API esi_status esi_synchronize(esi_ctx *ctx) {
+    if (!ctx) return ESI_ERR_ARG;
+    ctx->err.clear();
+    const esi_status e = check_dev_err(ctx);
+    for (size_t k = 0; e == ESI_OK && k < ctx->grp.size(); ++k)   // (the stream has waited for them)
+        if (const char *t = ctx->grp[k]->dev_err.text())
+            return ctx->fail(ESI_ERR_TIMEOUT, "shot group " + std::to_string(k) + ": " + t);
+    return e;
+}
 
 ESI_API esi_status esi_set_shot_groups(esi_ctx *ctx, int groups, const void *velocity_dev) {
     if (!ctx) return ESI_ERR_ARG;
@@ -3161,6 +3207,7 @@ ESI_API esi_status esi_set_shot_groups(esi_ctx *ctx, int groups, const void *vel
         }
         c->use_graphs = ctx->use_graphs;
         c->pdl = ctx->pdl;
+        c->loop_polls = ctx->loop_polls;
         c->prof = ctx->prof;
         ctx->grp.push_back(c);
         ctx->grp_s0.push_back(s0);
@@ -3191,7 +3238,7 @@ ESI_API esi_status esi_forward(esi_ctx *ctx, const void *wavelet_dev, const void
                                void *traces_dev) {
     if (!ctx) return ESI_ERR_ARG;
     if (!traces_dev) return ctx->fail(ESI_ERR_ARG, "traces_dev is NULL");
-    ctx->err.clear();
+    if (const esi_status e = begin_call(ctx)) return e;
     if (!ctx->grp.empty())
         return run_groups(ctx, [&](int k, esi_ctx *c) {
             const int s0 = ctx->grp_s0[k];
@@ -3207,7 +3254,7 @@ ESI_API esi_status esi_forward_noalloc(esi_ctx *ctx, const void *wavelet_dev,
                                        const void *ext_src_dev, void *traces_dev) {
     if (!ctx) return ESI_ERR_ARG;
     if (!traces_dev) return ctx->fail(ESI_ERR_ARG, "traces_dev is NULL");
-    ctx->err.clear();
+    if (const esi_status e = begin_call(ctx)) return e;
     return ctx->g.dtype == ESI_F64
                ? forward_noalloc_impl<double>(ctx, wavelet_dev, ext_src_dev, traces_dev)
                : forward_noalloc_impl<float>(ctx, wavelet_dev, ext_src_dev, traces_dev);
@@ -3218,7 +3265,7 @@ ESI_API esi_status esi_adjoint(esi_ctx *ctx, const void *traces_dev, void *ext_o
     if (!ctx) return ESI_ERR_ARG;
     if (!traces_dev || (!ext_out_dev && !wavelet_out_dev))
         return ctx->fail(ESI_ERR_ARG, "need adjoint data and at least one output");
-    ctx->err.clear();
+    if (const esi_status e = begin_call(ctx)) return e;
     if (!ctx->grp.empty())
         return run_groups(ctx, [&](int k, esi_ctx *c) {
             const int s0 = ctx->grp_s0[k];
@@ -3237,7 +3284,7 @@ ESI_API esi_status esi_gradient(esi_ctx *ctx, const void *wavelet_dev, const voi
     if (opts->param < ESI_PARAM_C || opts->param > ESI_PARAM_M ||
         opts->ckpt_kind < ESI_CKPT_F32 || opts->ckpt_kind > ESI_CKPT_BF16)
         return ctx->fail(ESI_ERR_ARG, "bad gradient options");
-    ctx->err.clear();
+    if (const esi_status e = begin_call(ctx)) return e;
     if (!ctx->grp.empty()) {
         // each group's gradient (the sum over its shots) into [G][N] scratch, then their sum
         const int G = (int)ctx->grp.size();
@@ -3276,7 +3323,7 @@ ESI_API esi_status esi_dft_extract(esi_ctx *ctx, const void *wavelet_dev, const 
                                    const double *freqs_hz, int nf, void *out_dev, int out_kind,
                                    float *scales_host, void *traces_dev) {
     if (!ctx) return ESI_ERR_ARG;
-    ctx->err.clear();
+    if (const esi_status e = begin_call(ctx)) return e;
     if (!ctx->grp.empty() && nf > 0) {
         const size_t cell = out_kind == ESI_DFT_C32_HALF ? 4 : 2 * (size_t)ctx->esz;
         return run_groups(ctx, [&](int k, esi_ctx *c) {
@@ -3301,7 +3348,7 @@ ESI_API esi_status esi_invert(esi_ctx *ctx, const esi_invert_opts *opts, const v
     if (!ctx) return ESI_ERR_ARG;
     if (!opts || !dobs_dev || !velocity_dev || !grad_dev)
         return ctx->fail(ESI_ERR_ARG, "bad outer-loop arguments");
-    ctx->err.clear();
+    if (const esi_status e = begin_call(ctx)) return e;
     return ctx->g.dtype == ESI_F64
                ? invert_impl<double>(ctx, opts, wavelet_dev, dobs_dev, velocity_dev, grad_dev, report)
                : invert_impl<float>(ctx, opts, wavelet_dev, dobs_dev, velocity_dev, grad_dev, report);
@@ -3314,7 +3361,7 @@ ESI_API esi_status esi_fdcg_solve(esi_ctx *ctx, double lambda, double tol, int m
     if (!ctx) return ESI_ERR_ARG;
     if (!dobs_dev || !qbar_out_dev || !freqs_hz || !(lambda > 0) || !(tol >= 0))
         return ctx->fail(ESI_ERR_ARG, "bad frequency-domain CG arguments");
-    ctx->err.clear();
+    if (const esi_status e = begin_call(ctx)) return e;
     if (!ctx->grp.empty() && nf >= 1)
         return run_group_solves(ctx, report, [&](int k, esi_ctx *c, esi_cg_report *r) {
             const int s0 = ctx->grp_s0[k];
@@ -3335,7 +3382,7 @@ ESI_API esi_status esi_dscg_solve(esi_ctx *ctx, double lambda, double tol, int m
     if (!ctx) return ESI_ERR_ARG;
     if (!dobs_dev || !q_out_dev || !(lambda > 0) || !(tol >= 0))
         return ctx->fail(ESI_ERR_ARG, "bad data-space CG arguments");
-    ctx->err.clear();
+    if (const esi_status e = begin_call(ctx)) return e;
     if (!ctx->grp.empty())
         return run_group_solves(ctx, report, [&](int k, esi_ctx *c, esi_cg_report *r) {
             const int s0 = ctx->grp_s0[k];
@@ -3356,7 +3403,7 @@ ESI_API esi_status esi_wri_solve(esi_ctx *ctx, double lambda, double tol, int ma
     if (!ctx) return ESI_ERR_ARG;
     if (!wavelet_dev || !dobs_dev || !q_out_dev || !(lambda >= 0) || !(tol >= 0))
         return ctx->fail(ESI_ERR_ARG, "bad WRI arguments");
-    ctx->err.clear();
+    if (const esi_status e = begin_call(ctx)) return e;
     if (!ctx->grp.empty())
         return run_group_solves(ctx, report, [&](int k, esi_ctx *c, esi_cg_report *r) {
             const int s0 = ctx->grp_s0[k];
@@ -3376,7 +3423,7 @@ ESI_API esi_status esi_cg_solve(esi_ctx *ctx, double lambda, double tol, int max
     if (!ctx) return ESI_ERR_ARG;
     if (!dobs_dev || !q_out_dev || !(lambda >= 0) || !(tol >= 0))
         return ctx->fail(ESI_ERR_ARG, "bad CG arguments");
-    ctx->err.clear();
+    if (const esi_status e = begin_call(ctx)) return e;
     if (!ctx->grp.empty() && precond != ESI_PC_LEARNED) {
         // the network's buffers belong to this context: the learned solve runs here
         return run_group_solves(ctx, report, [&](int k, esi_ctx *c, esi_cg_report *r) {
@@ -3400,7 +3447,8 @@ ESI_API esi_status esi_pc_load(esi_ctx *ctx, const void *weights_dev, size_t byt
         const long long nimg = (long long)ctx->ns * ((ctx->nt + 15) / 16);
         ctx->pc_batch = (int)std::min<long long>(nimg, 512);
         std::string err;
-        ctx->pc = pcnet_create((ctx->g.nz + 1) / 2, (ctx->g.nx + 1) / 2, ctx->pc_batch, ctx->st, &err);
+        ctx->pc = pcnet_create((ctx->g.nz + 1) / 2, (ctx->g.nx + 1) / 2, ctx->pc_batch, ctx->dev_err.d,
+                               ctx->st, &err);
         if (!ctx->pc) return ctx->fail(ESI_ERR_OOM, err);
     }
     CK(pcnet_set_params(ctx->pc, reinterpret_cast<const float *>(weights_dev), ctx->st));
@@ -3413,7 +3461,7 @@ ESI_API esi_status esi_normal_apply(esi_ctx *ctx, double lambda, double eps, con
                                     void *out_dev) {
     if (!ctx) return ESI_ERR_ARG;
     if (!p_dev || !out_dev || !(lambda >= 0)) return ctx->fail(ESI_ERR_ARG, "bad arguments");
-    ctx->err.clear();
+    if (const esi_status e = begin_call(ctx)) return e;
     if (!ctx->grp.empty())
         return run_groups(ctx, [&](int k, esi_ctx *c) {
             const int s0 = ctx->grp_s0[k];

@@ -168,6 +168,18 @@ struct StepArgs {
 // device error codes written to StepArgs::dev_err
 constexpr int DEV_ERR_TMA_TIMEOUT = 1;
 constexpr int DEV_ERR_LOOP_TIMEOUT = 2;
+// The sticky error word of a context or network, in mapped host memory: a kernel whose bounded
+// wait runs out writes it, and the host reads it without a call or a synchronisation, so that a
+// call that only enqueues can tell what became of the ones before it.
+struct ErrWord {
+    int *h = nullptr, *d = nullptr;   // its host and device address
+    ErrWord() = default;
+    ErrWord(const ErrWord &) = delete;
+    ErrWord &operator=(const ErrWord &) = delete;
+    ~ErrWord();
+    cudaError_t make();
+    const char *text() const;   // what the word says, or NULL
+};
 // iteration limit of the mbarrier wait for a TMA tile (a tile arrives in microseconds;
 // the limit is seconds of polling)
 constexpr long long TMA_WAIT_LIMIT = 1ll << 26;
@@ -188,6 +200,7 @@ int step3_chunks(int nz, long long cols, int esz);
 // cell blocks, a tile is a range of block columns x a range of block rows.
 constexpr int LOOP_THREADS = 512;        // compute + communication threads, at most
 constexpr int LOOP_COMM = 128;           // communication threads
+constexpr int LOOP_POLLS = 1 << 22;      // of a rim packet (about 0.6 us each: seconds)
 constexpr int LOOP_SMEM = 226 * 1024;    // dynamic shared memory of a tile, at most
 
 // first block of part i when n blocks are cut into `parts` near-equal ranges
@@ -222,6 +235,7 @@ struct LoopArgs {
     int gx, gz;              // tiles per shot along x and z
     int qx, gr;              // block columns and block rows of the plane
     int steps, dn;           // time steps; increment (+1 / -1) of every time index per step
+    int polls;               // of a packet, before a wait gives up
     int nt;                  // traces are sampled at 0 <= tout < nt
     int nc, nm;              // compute and communication threads
     int lanes;               // lanes along x per group of compute threads

@@ -87,7 +87,8 @@ cudaError_t pc_dots_launch(const float *r, const float *ap, const float *ipb2, c
 
 // The network object used by the C ABI and by the preconditioned CG.
 struct PcNet;
-PcNet *pcnet_create(int H1, int W1, int max_batch, cudaStream_t st, std::string *err);
+// (err_word: the owner's ErrWord on the device)
+PcNet *pcnet_create(int H1, int W1, int max_batch, int *err_word, cudaStream_t st, std::string *err);
 void pcnet_destroy(PcNet *p);
 cudaError_t pcnet_set_params(PcNet *p, const float *params_dev, cudaStream_t st);
 cudaError_t pcnet_get_params(const PcNet *p, float *params_dev, cudaStream_t st);
@@ -106,6 +107,5 @@ cudaError_t pcnet_grad(PcNet *p, const __nv_bfloat16 *x, const __nv_bfloat16 *e,
 cudaError_t pcnet_vjp(PcNet *p, const __nv_bfloat16 *x, const float *gy, int n, float *grad_out,
                       cudaStream_t st);
 cudaError_t pcnet_adam(PcNet *p, double lr, cudaStream_t st);
-int *pcnet_dev_err(PcNet *p);
 
 }  // namespace esi

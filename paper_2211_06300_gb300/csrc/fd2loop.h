@@ -38,8 +38,6 @@ namespace loop2 {
 
 constexpr double W0 = -205.0 / 72.0, W1 = 8.0 / 5.0, W2 = -1.0 / 5.0, W3 = 8.0 / 315.0,
                  W4 = -1.0 / 560.0;
-// polls of a packet before a wait gives up (about 0.6 us each: seconds)
-constexpr int POLL_LIMIT = 1 << 22;
 constexpr int SMP_T = 32;     // of the communication threads: those that sample the receivers
 constexpr int INJ_U = 4;      // trace values a thread has in flight for the point sources
 constexpr int PF_AHEAD = 2;   // steps by which the streams' L2 prefetch runs ahead
@@ -635,7 +633,7 @@ __global__ void __launch_bounds__(LOOP_THREADS, 1)
                                         unpack(v[u], B + dst[u]);
                                         open &= ~(1u << u);
                                     }
-                                if (polls >= POLL_LIMIT) {
+                                if (polls >= g.polls) {
                                     atomicExch(a.dev_err, DEV_ERR_LOOP_TIMEOUT);
                                     late = true;
                                     break;

@@ -45,7 +45,7 @@ struct PcNet {
     Buf gy, gL1, gD2, gL2, gD3, gL3, gBT, gP3, gP2, gP1, gbf, dwpart, yscratch, dots;
     Buf xn, rms;    // normalised input images and their per-image scale
     Buf rms_acc;    // per-image FP64 sums of squares
-    Buf dev_err;
+    int *dev_err = nullptr;   // the owner's error word
     bool weights_ready = false;
 };
 
@@ -80,13 +80,14 @@ const float *bias_of(const PcNet *p, int l) {
 
 }  // namespace
 
-PcNet *pcnet_create(int H1, int W1, int max_batch, cudaStream_t st, std::string *err) {
+PcNet *pcnet_create(int H1, int W1, int max_batch, int *err_word, cudaStream_t st, std::string *err) {
     if (H1 < 1 || W1 < 1 || max_batch < 1) {
         *err = "bad preconditioner size";
         return nullptr;
     }
     PcNet *p = new PcNet();
     p->max_batch = max_batch;
+    p->dev_err = err_word;
     p->H[0] = H1;
     p->W[0] = W1;
     for (int l = 1; l < 4; ++l) {
@@ -113,7 +114,7 @@ PcNet *pcnet_create(int H1, int W1, int max_batch, cudaStream_t st, std::string 
         (e = act(p->p2, 2, C)) || (e = act(p->e3, 2, C)) || (e = act(p->p3, 3, C)) ||
         (e = act(p->bt, 3, C)) || (e = act(p->u3, 2, C)) || (e = act(p->d3, 2, C)) ||
         (e = act(p->u2, 1, C)) || (e = act(p->d2, 1, C)) || (e = act(p->u1, 0, C)) ||
-        (e = p->dev_err.ensure(sizeof(int))) || (e = p->dots.ensure(sizeof(double) * 3 * n)) ||
+        (e = p->dots.ensure(sizeof(double) * 3 * n)) ||
         (e = act(p->xn, 0, G)) || (e = p->rms.ensure(sizeof(float) * n)) ||
         (e = p->rms_acc.ensure(sizeof(double) * n))) {
         *err = std::string("preconditioner allocation: ") + cudaGetErrorString(e);
@@ -123,13 +124,10 @@ PcNet *pcnet_create(int H1, int W1, int max_batch, cudaStream_t st, std::string 
     cudaMemsetAsync(p->params.p, 0, np, st);
     cudaMemsetAsync(p->m.p, 0, np, st);
     cudaMemsetAsync(p->v.p, 0, np, st);
-    cudaMemsetAsync(p->dev_err.p, 0, sizeof(int), st);
     return p;
 }
 
 void pcnet_destroy(PcNet *p) { delete p; }
-
-int *pcnet_dev_err(PcNet *p) { return p->dev_err.as<int>(); }
 
 cudaError_t pcnet_set_params(PcNet *p, const float *src, cudaStream_t st) {
     RET(cudaMemcpyAsync(p->params.p, src, (size_t)param_count() * 4, cudaMemcpyDeviceToDevice, st));
@@ -148,7 +146,7 @@ cudaError_t pcnet_forward(PcNet *p, const __nv_bfloat16 *x, int n, float *y, cud
     if (n > p->max_batch || n < 1) return cudaErrorInvalidValue;
     if (!p->weights_ready) RET(prep_weights(p, st));
     const int *H = p->H, *W = p->W;
-    int *de = p->dev_err.as<int>();
+    int *de = p->dev_err;
     auto wf = [&](int l) { return p->wf.as<__nv_bfloat16>() + p->wf_off[l]; };
     using bf = __nv_bfloat16;
     RET(normalize_launch(x, p->rms.as<float>(), p->rms_acc.as<double>(), keep_xn ? p->xn.as<bf>() : nullptr, n,
@@ -216,7 +214,7 @@ cudaError_t backward_from_gy(PcNet *p, int n, cudaStream_t st) {
     // y = rms * U(xn): the network's output gradient carries the per-image scale
     RET(img_mul_launch(p->gy.as<float>(), p->rms.as<float>(), n, (long long)H[0] * W[0] * G, st));
     const bf *xin = p->xn.as<bf>();   // the first layer saw the normalised images
-    int *de = p->dev_err.as<int>();
+    int *de = p->dev_err;
     auto wb = [&](int l) { return p->wb.as<__nv_bfloat16>() + p->wf_off[l]; };
     auto gW = [&](int l) { return p->grads.as<float>() + p->off[l]; };
     auto gB = [&](int l) { return p->grads.as<float>() + p->off[l] + 9ll * LAYERS[l].cin * LAYERS[l].cout; };
@@ -316,6 +314,7 @@ cudaError_t pcnet_adam(PcNet *p, double lr, cudaStream_t st) {
 
 // ----------------------------------------------------------------------------- C ABI
 struct esi_pc {
+    esi::ErrWord dev_err;
     esi::PcNet *net = nullptr;
     cudaStream_t st = nullptr;
     std::string err;
@@ -329,16 +328,17 @@ esi_status pc_fail(esi_pc *pc, cudaError_t e, const char *what) {
     return e == cudaErrorMemoryAllocation ? ESI_ERR_OOM : ESI_ERR_CUDA;
 }
 
+// what the sticky error word says so far; the same after the work queued on the stream
+esi_status pc_err_status(esi_pc *pc) {
+    const char *t = pc->dev_err.text();
+    if (!t) return ESI_OK;
+    pc->err = t;
+    return ESI_ERR_TIMEOUT;
+}
 esi_status pc_check_err(esi_pc *pc) {
-    int h = 0;
-    cudaMemcpyAsync(&h, esi::pcnet_dev_err(pc->net), sizeof(int), cudaMemcpyDeviceToHost, pc->st);
     cudaError_t e = cudaStreamSynchronize(pc->st);
     if (e != cudaSuccess) return pc_fail(pc, e, "preconditioner");
-    if (h) {
-        pc->err = "a tensor-core tile wait ran out of its iteration limit";
-        return ESI_ERR_TIMEOUT;
-    }
-    return ESI_OK;
+    return pc_err_status(pc);
 }
 }  // namespace
 
@@ -352,7 +352,9 @@ ESI_API esi_status esi_pc_create(esi_pc **out, int h, int w, int max_batch, void
     *out = nullptr;
     esi_pc *pc = new esi_pc();
     pc->st = reinterpret_cast<cudaStream_t>(stream);
-    pc->net = esi::pcnet_create(h, w, max_batch, pc->st, &g_pc_create_error);
+    const cudaError_t ce = pc->dev_err.make();
+    if (ce != cudaSuccess) g_pc_create_error = std::string("preconditioner allocation: ") + cudaGetErrorString(ce);
+    else pc->net = esi::pcnet_create(h, w, max_batch, pc->dev_err.d, pc->st, &g_pc_create_error);
     if (!pc->net) {
         delete pc;
         return ESI_ERR_OOM;
@@ -386,6 +388,7 @@ ESI_API esi_status esi_pc_get_params(esi_pc *pc, float *params_dev) {
 
 ESI_API esi_status esi_pc_apply(esi_pc *pc, const void *in_dev, int n, float *y_dev) {
     if (!pc || !in_dev || !y_dev || n < 1) return ESI_ERR_ARG;
+    if (const esi_status st = pc_err_status(pc)) return st;
     cudaError_t e = esi::pcnet_forward(pc->net, reinterpret_cast<const __nv_bfloat16 *>(in_dev), n,
                                        y_dev, pc->st);
     if (e != cudaSuccess) return pc_fail(pc, e, "apply");
@@ -395,6 +398,7 @@ ESI_API esi_status esi_pc_apply(esi_pc *pc, const void *in_dev, int n, float *y_
 ESI_API esi_status esi_pc_grad(esi_pc *pc, const void *in_dev, const void *target_dev, int n,
                                float *grad_dev, double *loss) {
     if (!pc || !in_dev || !target_dev || n < 1) return ESI_ERR_ARG;
+    if (const esi_status st = pc_err_status(pc)) return st;
     cudaError_t e = esi::pcnet_grad(pc->net, reinterpret_cast<const __nv_bfloat16 *>(in_dev),
                                     reinterpret_cast<const __nv_bfloat16 *>(target_dev), n, loss,
                                     grad_dev, pc->st);
@@ -405,6 +409,7 @@ ESI_API esi_status esi_pc_grad(esi_pc *pc, const void *in_dev, const void *targe
 ESI_API esi_status esi_pc_vjp(esi_pc *pc, const void *in_dev, const float *gy_dev, int n,
                               float *grad_dev) {
     if (!pc || !in_dev || !gy_dev || !grad_dev || n < 1) return ESI_ERR_ARG;
+    if (const esi_status st = pc_err_status(pc)) return st;
     cudaError_t e = esi::pcnet_vjp(pc->net, reinterpret_cast<const __nv_bfloat16 *>(in_dev), gy_dev,
                                    n, grad_dev, pc->st);
     if (e != cudaSuccess) return pc_fail(pc, e, "vjp");
@@ -414,6 +419,7 @@ ESI_API esi_status esi_pc_vjp(esi_pc *pc, const void *in_dev, const float *gy_de
 ESI_API esi_status esi_pc_train_step(esi_pc *pc, const void *in_dev, const void *target_dev, int n,
                                      double lr, double *loss) {
     if (!pc || !in_dev || !target_dev || n < 1 || !(lr > 0)) return ESI_ERR_ARG;
+    if (const esi_status st = pc_err_status(pc)) return st;
     cudaError_t e = esi::pcnet_grad(pc->net, reinterpret_cast<const __nv_bfloat16 *>(in_dev),
                                     reinterpret_cast<const __nv_bfloat16 *>(target_dev), n, loss,
                                     nullptr, pc->st);

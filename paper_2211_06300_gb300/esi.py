@@ -33,7 +33,7 @@ EXPORTS = ["esi_create", "esi_destroy", "esi_set_stream", "esi_set_velocity", "e
            "esi_pc_fallbacks", "esi_pc_pack", "esi_pc_create", "esi_pc_destroy",
            "esi_pc_last_error", "esi_pc_set_params", "esi_pc_get_params", "esi_pc_apply",
            "esi_pc_grad", "esi_pc_vjp", "esi_pc_train_step", "esi_wri_solve", "esi_dscg_solve",
-           "esi_fdcg_solve", "esi_invert", "esi_set_shot_groups"]
+           "esi_fdcg_solve", "esi_invert", "esi_set_shot_groups", "esi_synchronize"]
 
 
 class EsiGrid(ctypes.Structure):
@@ -120,6 +120,7 @@ def load_library(require_gpu: bool = True) -> ctypes.CDLL:
     L.esi_destroy.argtypes = [vp]
     L.esi_destroy.restype = None
     L.esi_set_stream.argtypes = [vp, vp]
+    L.esi_synchronize.argtypes = [vp]
     L.esi_set_velocity.argtypes = [vp, vp]
     L.esi_set_shot_groups.argtypes = [vp, i, vp]
     L.esi_forward.argtypes = [vp, vp, vp, vp]
@@ -170,7 +171,7 @@ def load_library(require_gpu: bool = True) -> ctypes.CDLL:
                  "esi_pc_vjp", "esi_pc_train_step",
                  "esi_adjoint", "esi_gradient", "esi_dft_extract", "esi_cg_solve",
                  "esi_pc_load", "esi_wri_solve", "esi_dscg_solve", "esi_fdcg_solve", "esi_invert",
-                 "esi_set_shot_groups"):
+                 "esi_set_shot_groups", "esi_synchronize"):
         getattr(L, name).restype = ctypes.c_int
     _lib = L
     return L
@@ -294,6 +295,10 @@ class Context:
         return [{"name": arr[i].name.decode(), "launches": int(arr[i].launches),
                  "cells": int(arr[i].cells), "bytes_per_cell": float(arr[i].bytes_per_cell),
                  "ms": float(arr[i].ms)} for i in range(n)]
+
+    def synchronize(self):
+        """Wait for the context's work; raises when a device wait of it ran out (esi_synchronize)."""
+        self._check(self.L.esi_synchronize(self.h))
 
     # ---------------------------------------------------------------- operators
     def set_velocity(self, v):
