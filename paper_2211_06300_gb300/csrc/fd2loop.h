@@ -299,23 +299,25 @@ __global__ void __launch_bounds__(LOOP_THREADS, 1)
         // per cell adds them up from shared memory.  (2000 receivers on a line, back-propagation, us
         // per step, with one load at a time by the cell's thread and so: one shot of 101 x 101 33 and
         // 3.0, 20 shots of 97 x 130 68 and 4.9; the per-step kernel 7.7 and 8.1.)
-        bool several = false;
+        const bool several = nci > 0 && inj[nci - 1].pos == LOOP_NONE;
         auto inject = [&](T *p, int t, int me, int n, auto &&sync) {
-            for (int c0 = me; c0 < nci; c0 += INJ_U * n) {
-                T v[INJ_U];
+            auto load = [&](int c) { return a.inj_trace[inj[c].off + (long long)t * inj[c].stride]; };
+            auto place = [&](int c, T v) {
+                T sum = T(0);
+                sum += inj[c].w * v;
+                if (several) inj[c].v = v;
+                else p[inj[c].pos] = sum;
+            };
+            if (nci <= n) {
+                if (me < nci) place(me, load(me));
+            } else {
+                for (int c0 = me; c0 < nci; c0 += INJ_U * n) {
+                    T v[INJ_U];
 #pragma unroll
-                for (int u = 0; u < INJ_U; ++u) {
-                    const int c = c0 + u * n;
-                    v[u] = c < nci ? a.inj_trace[inj[c].off + (long long)t * inj[c].stride] : T(0);
-                }
+                    for (int u = 0; u < INJ_U; ++u) v[u] = c0 + u * n < nci ? load(c0 + u * n) : T(0);
 #pragma unroll
-                for (int u = 0; u < INJ_U; ++u) {
-                    const int c = c0 + u * n;
-                    if (c >= nci) break;
-                    T sum = T(0);
-                    sum += inj[c].w * v[u];
-                    if (several) inj[c].v = v[u];
-                    else p[inj[c].pos] = sum;
+                    for (int u = 0; u < INJ_U; ++u)
+                        if (c0 + u * n < nci) place(c0 + u * n, v[u]);
                 }
             }
             if (!several) return;
@@ -329,8 +331,6 @@ __global__ void __launch_bounds__(LOOP_THREADS, 1)
             }
         };
         if constexpr ((F & F_PT) != 0) {
-            if (tid == 0 && nci > 0) several = inj[nci - 1].pos == LOOP_NONE;
-            several = __syncthreads_or(several);
             inject(patch, a.tin, tid, nthr, [] { __syncthreads(); });
             __syncthreads();
         }
