@@ -32,6 +32,7 @@
 #include <type_traits>
 
 #include "esi_internal.h"
+#include "pairs.h"
 
 namespace esi {
 namespace loop2 {
@@ -42,9 +43,8 @@ constexpr int SMP_T = 32;     // of the communication threads: those that sample
 constexpr int INJ_U = 4;      // trace values a thread has in flight for the point sources
 constexpr int PF_AHEAD = 2;   // steps by which the streams' L2 prefetch runs ahead
 
-// The cells of one thread along x: four FP32 as two packed pairs (f32x2 instructions halve the
-// issue slots of the stencil's arithmetic; each lane rounds as the scalar instruction does), or
-// one FP64.
+// The cells of one thread along x: four FP32 as two pairs in the arithmetic of the step kernels
+// (pairs.h; each lane rounds as the scalar instruction does), or one FP64.
 template <typename T>
 struct Row4;
 template <>
@@ -58,42 +58,21 @@ struct Row4<double> {
     double p[1];
 };
 
+using PF = Pk<float>;
 __device__ __forceinline__ unsigned long long pack2(float x, float y) {
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-    return r;
+    const float v[2] = {x, y};
+    return PF::pack(v);
 }
 __device__ __forceinline__ float lo2(unsigned long long v) { return __uint_as_float((unsigned)v); }
 __device__ __forceinline__ float hi2(unsigned long long v) { return __uint_as_float((unsigned)(v >> 32)); }
-__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
-    unsigned long long r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ unsigned long long sub2(unsigned long long a, unsigned long long b) {
-    unsigned long long r;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
-    unsigned long long r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b,
-                                                   unsigned long long c) {
-    unsigned long long r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
 
 using RF = Row4<float>;
 using RD = Row4<double>;
-__device__ __forceinline__ RF add(const RF &a, const RF &b) { return {{add2(a.p[0], b.p[0]), add2(a.p[1], b.p[1])}}; }
-__device__ __forceinline__ RF sub(const RF &a, const RF &b) { return {{sub2(a.p[0], b.p[0]), sub2(a.p[1], b.p[1])}}; }
-__device__ __forceinline__ RF mul(const RF &a, const RF &b) { return {{mul2(a.p[0], b.p[0]), mul2(a.p[1], b.p[1])}}; }
+__device__ __forceinline__ RF add(const RF &a, const RF &b) { return {{PF::add(a.p[0], b.p[0]), PF::add(a.p[1], b.p[1])}}; }
+__device__ __forceinline__ RF sub(const RF &a, const RF &b) { return {{PF::sub(a.p[0], b.p[0]), PF::sub(a.p[1], b.p[1])}}; }
+__device__ __forceinline__ RF mul(const RF &a, const RF &b) { return {{PF::mul(a.p[0], b.p[0]), PF::mul(a.p[1], b.p[1])}}; }
 __device__ __forceinline__ RF fma(const RF &a, const RF &b, const RF &c) {
-    return {{fma2(a.p[0], b.p[0], c.p[0]), fma2(a.p[1], b.p[1], c.p[1])}};
+    return {{PF::fma(a.p[0], b.p[0], c.p[0]), PF::fma(a.p[1], b.p[1], c.p[1])}};
 }
 __device__ __forceinline__ RF splat(float v) { return {{pack2(v, v), pack2(v, v)}}; }
 __device__ __forceinline__ float at(const RF &a, int i) { return (i & 1) ? hi2(a.p[i >> 1]) : lo2(a.p[i >> 1]); }
@@ -128,7 +107,7 @@ struct Side<float> {
     template <int D>
     __device__ __forceinline__ RF sum(const RF &c) const {
         if constexpr (D == 4) return add(l, r);
-        if constexpr (D == 2) return {{add2(l.p[1], c.p[1]), add2(c.p[0], r.p[0])}};
+        if constexpr (D == 2) return {{PF::add(l.p[1], c.p[1]), PF::add(c.p[0], r.p[0])}};
         if constexpr (D == 1)
             return {{pack2(hi2(l.p[1]) + hi2(c.p[0]), lo2(c.p[0]) + lo2(c.p[1])),
                      pack2(hi2(c.p[0]) + hi2(c.p[1]), lo2(c.p[1]) + lo2(r.p[0]))}};
