@@ -704,6 +704,16 @@ esi_status idft_block_chains(esi_ctx *ctx, const T *qb, int K, int kst, int nf, 
     return ESI_OK;
 }
 
+// alpha c of the model and sponge, which only the on-chip loops read
+template <typename T>
+esi_status setup_alpha(esi_ctx *ctx) {
+    if (!ctx->lp.ok) return ESI_OK;
+    CK(ctx->ac.ensure(ctx->sst * sizeof(T)));
+    CKL(launch_alpha_c<T>(ctx->cc.as<T>(), ctx->kz.as<T>(), ctx->kx.as<T>(), ctx->ac.as<T>(),
+                          ctx->g.nz, ctx->px, ctx->st));
+    return ESI_OK;
+}
+
 template <typename T>
 esi_status setup_model(esi_ctx *ctx, const void *vel, bool first) {
     const int nblk = 1024;
@@ -754,12 +764,7 @@ esi_status setup_model(esi_ctx *ctx, const void *vel, bool first) {
         // padded to the x pitch (zeros) for 16-byte loads
         CK(upload(ctx->kx, prof(ctx->g.nx, true, ctx->px), ctx->st));
     }
-    if (ctx->g.ndim == 2) {
-        CK(ctx->ac.ensure(ctx->sst * sizeof(T)));
-        CKL(launch_alpha_c<T>(ctx->cc.as<T>(), ctx->kz.as<T>(), ctx->kx.as<T>(), ctx->ac.as<T>(),
-                              ctx->g.nz, ctx->px, ctx->st));
-    }
-    return ESI_OK;
+    return setup_alpha<T>(ctx);
 }
 
 // ------------------------------------------------------------------ plan of the on-chip loops
@@ -1076,6 +1081,7 @@ esi_status setup_geometry(esi_ctx *ctx) {
     if ((e = build_smp<T>(ctx, ctx->smp_rec, rec_smp)) != ESI_OK) return e;
     if ((e = build_smp<T>(ctx, ctx->smp_src, src_smp)) != ESI_OK) return e;
     if ((e = setup_loops<T>(ctx, src_inj, rec_inj, rec_smp, src_smp)) != ESI_OK) return e;
+    if ((e = setup_alpha<T>(ctx)) != ESI_OK) return e;   // (a new model: setup_model)
     if ((e = setup_chains<T>(ctx)) != ESI_OK) return e;
     CK(upload(ctx->src_pos, ctx->src_xyz, ctx->st));
     return ESI_OK;

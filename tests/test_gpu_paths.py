@@ -35,3 +35,28 @@ def test_the_path_of_a_time_loop(nz, nx, ns, dtype, per_step):
     else:
         assert n <= ns + 1
     c.close()
+
+
+@pytest.mark.parametrize("nz,nx,ns,dtype,per_step", [(45, 83, 3, F32, 0), (45, 83, 3, F64, 0),
+                                                     (241, 801, 4, F32, 1), (241, 801, 7, F32, 2)])
+def test_a_new_model_reaches_the_loops_and_costs_what_they_use(nz, nx, ns, dtype, per_step):
+    """alpha c, which only the on-chip loops read, is worked out for contexts that have them: at
+    creation and for every new model (the model's own kernel is the other launch)."""
+    from paper_2211_06300_gb300 import esi
+    nt = 40
+    geom = synth.surface_line(ns, np.linspace(0.0, (nx - 1) * 10.0, ns), 20.0,
+                              [np.linspace(0.0, (nx - 1) * 10.0, 5)] * ns, 20.0)
+    rng = np.random.default_rng(nx)
+    v = [torch.tensor(1500.0 + 1000.0 * rng.random((nz, nx)), dtype=dtype, device="cuda") for _ in range(2)]
+    wav = torch.tensor(rng.standard_normal((ns, nt)), dtype=dtype, device="cuda")
+    a, b = [esi.Context(x, 10.0, 1e-3, nt, 2, geom, vref=2500.0) for x in v]
+    n = 1 if per_step else 2
+    assert a.launches == n
+    first = a.forward(wavelet=wav)
+    n0 = a.launches
+    a.set_velocity(v[1])
+    assert a.launches - n0 == n
+    second = a.forward(wavelet=wav)
+    assert torch.equal(second, b.forward(wavelet=wav)) and not torch.equal(first, second)
+    a.close()
+    b.close()
