@@ -3453,8 +3453,8 @@ ESI_API esi_status esi_pc_load(esi_ctx *ctx, const void *weights_dev, size_t byt
         const long long nimg = (long long)ctx->ns * ((ctx->nt + 15) / 16);
         ctx->pc_batch = (int)std::min<long long>(nimg, 512);
         std::string err;
-        ctx->pc = pcnet_create((ctx->g.nz + 1) / 2, (ctx->g.nx + 1) / 2, ctx->pc_batch, ctx->dev_err.d,
-                               ctx->st, &err);
+        ctx->pc = pcnet_create((ctx->g.nz + 1) / 2, (ctx->g.nx + 1) / 2, ctx->pc_batch, false,
+                               ctx->dev_err.d, ctx->st, &err);
         if (!ctx->pc) return ctx->fail(ESI_ERR_OOM, err);
     }
     CK(pcnet_set_params(ctx->pc, reinterpret_cast<const float *>(weights_dev), ctx->st));

@@ -87,8 +87,10 @@ cudaError_t pc_dots_launch(const float *r, const float *ap, const float *ipb2, c
 
 // The network object used by the C ABI and by the preconditioned CG.
 struct PcNet;
-// (err_word: the owner's ErrWord on the device)
-PcNet *pcnet_create(int H1, int W1, int max_batch, int *err_word, cudaStream_t st, std::string *err);
+// err_word: the owner's ErrWord on the device; train: with the buffers that only gradients need
+// (a CG's network is applied, never trained)
+PcNet *pcnet_create(int H1, int W1, int max_batch, bool train, int *err_word, cudaStream_t st,
+                    std::string *err);
 void pcnet_destroy(PcNet *p);
 cudaError_t pcnet_set_params(PcNet *p, const float *params_dev, cudaStream_t st);
 cudaError_t pcnet_get_params(const PcNet *p, float *params_dev, cudaStream_t st);

@@ -80,7 +80,8 @@ const float *bias_of(const PcNet *p, int l) {
 
 }  // namespace
 
-PcNet *pcnet_create(int H1, int W1, int max_batch, int *err_word, cudaStream_t st, std::string *err) {
+PcNet *pcnet_create(int H1, int W1, int max_batch, bool train, int *err_word, cudaStream_t st,
+                    std::string *err) {
     if (H1 < 1 || W1 < 1 || max_batch < 1) {
         *err = "bad preconditioner size";
         return nullptr;
@@ -112,11 +113,12 @@ PcNet *pcnet_create(int H1, int W1, int max_batch, int *err_word, cudaStream_t s
         (e = p->v.ensure(np)) || (e = p->wf.ensure(wo * 2)) || (e = p->wb.ensure(wo * 2)) ||
         (e = act(p->e1, 0, C)) || (e = act(p->p1, 1, C)) || (e = act(p->e2, 1, C)) ||
         (e = act(p->p2, 2, C)) || (e = act(p->e3, 2, C)) || (e = act(p->p3, 3, C)) ||
-        (e = act(p->bt, 3, C)) || (e = act(p->u3, 2, C)) || (e = act(p->d3, 2, C)) ||
-        (e = act(p->u2, 1, C)) || (e = act(p->d2, 1, C)) || (e = act(p->u1, 0, C)) ||
-        (e = p->dots.ensure(sizeof(double) * 3 * n)) ||
-        (e = act(p->xn, 0, G)) || (e = p->rms.ensure(sizeof(float) * n)) ||
-        (e = p->rms_acc.ensure(sizeof(double) * n))) {
+        (e = act(p->bt, 3, C)) || (e = act(p->d3, 2, C)) || (e = act(p->d2, 1, C)) ||
+        (e = p->dots.ensure(sizeof(double) * 3 * n)) || (e = p->rms.ensure(sizeof(float) * n)) ||
+        (e = p->rms_acc.ensure(sizeof(double) * n)) ||
+        // the decoder's sums and the normalised input, as the weight gradient reads them
+        (train && ((e = act(p->u3, 2, C)) || (e = act(p->u2, 1, C)) || (e = act(p->u1, 0, C)) ||
+                   (e = act(p->xn, 0, G))))) {
         *err = std::string("preconditioner allocation: ") + cudaGetErrorString(e);
         delete p;
         return nullptr;
@@ -354,7 +356,7 @@ ESI_API esi_status esi_pc_create(esi_pc **out, int h, int w, int max_batch, void
     pc->st = reinterpret_cast<cudaStream_t>(stream);
     const cudaError_t ce = pc->dev_err.make();
     if (ce != cudaSuccess) g_pc_create_error = std::string("preconditioner allocation: ") + cudaGetErrorString(ce);
-    else pc->net = esi::pcnet_create(h, w, max_batch, pc->dev_err.d, pc->st, &g_pc_create_error);
+    else pc->net = esi::pcnet_create(h, w, max_batch, true, pc->dev_err.d, pc->st, &g_pc_create_error);
     if (!pc->net) {
         delete pc;
         return ESI_ERR_OOM;
