@@ -272,37 +272,64 @@ __global__ void __launch_bounds__(LOOP_THREADS, 1)
         }
         __syncthreads();
         // The point-source cells at trace time t into the patch set p, by the `n` threads that call
-        // this as me = 0 .. n - 1.  A cell's contributions (usually one) are added in list order.
-        // Loads of a thread's entries go out INJ_U at a time: an entry is the latency of L2 or HBM,
-        // and a tile can hold thousands.  Where a cell has several, all threads load, and a thread
-        // per cell adds them up from shared memory.  (2000 receivers on a line, back-propagation, us
-        // per step, with one load at a time by the cell's thread and so: one shot of 101 x 101 33 and
-        // 3.0, 20 shots of 97 x 130 68 and 4.9; the per-step kernel 7.7 and 8.1.)
+        // this as me = 0 .. n - 1.  A cell's contributions are added in list order.  An entry is the
+        // latency of L2 or HBM, so a thread's loads go out together.  Short lists (a cell a thread,
+        // up to INJ_U contributions each) go straight to the cells.  Of long ones, which can hold
+        // thousands of entries a tile, all threads load entries, INJ_U at a time each; where a cell
+        // has several contributions, a thread per cell then adds them up from shared memory.  (2000
+        // receivers on a line, back-propagation, us per step, with one load at a time by the cell's
+        // thread and so: one shot of 101 x 101 33 and 3.0, 20 shots of 97 x 130 68 and 4.9; the
+        // per-step kernel 7.7 and 8.1.)
         const bool several = nci > 0 && inj[nci - 1].pos == LOOP_NONE;
+        auto end_of = [&](int i) {
+            return i + 1 < nci && inj[i + 1].pos != LOOP_NONE ? (int)inj[i + 1].first : nci;
+        };
+        bool longer = nci > g.nm - SMP_T && inj[g.nm - SMP_T].pos != LOOP_NONE;
+        if (several) {
+            bool chain = false;
+            for (int i = tid; i < nci && inj[i].pos != LOOP_NONE; i += nthr)
+                chain |= end_of(i) - inj[i].first > INJ_U;
+            longer |= __syncthreads_or(chain) != 0;
+        }
+        auto load = [&](int c, int t) { return a.inj_trace[inj[c].off + (long long)t * inj[c].stride]; };
         auto inject = [&](T *p, int t, int me, int n, auto &&sync) {
-            auto load = [&](int c) { return a.inj_trace[inj[c].off + (long long)t * inj[c].stride]; };
-            auto place = [&](int c, T v) {
-                T sum = T(0);
-                sum += inj[c].w * v;
-                if (several) inj[c].v = v;
-                else p[inj[c].pos] = sum;
-            };
-            if (nci <= n) {
-                if (me < nci) place(me, load(me));
-            } else {
-                for (int c0 = me; c0 < nci; c0 += INJ_U * n) {
-                    T v[INJ_U];
+            if (!longer) {
+                if (me >= nci || inj[me].pos == LOOP_NONE) return;
+                const int c = several ? inj[me].first : me;
+                T v[INJ_U], sum = T(0);
+                v[0] = load(c, t);
+                if (several) {
+                    const int end = end_of(me);
 #pragma unroll
-                    for (int u = 0; u < INJ_U; ++u) v[u] = c0 + u * n < nci ? load(c0 + u * n) : T(0);
+                    for (int u = 1; u < INJ_U; ++u) v[u] = c + u < end ? load(c + u, t) : T(0);
+                    sum += inj[c].w * v[0];
 #pragma unroll
-                    for (int u = 0; u < INJ_U; ++u)
-                        if (c0 + u * n < nci) place(c0 + u * n, v[u]);
+                    for (int u = 1; u < INJ_U; ++u)
+                        if (c + u < end) sum += inj[c + u].w * v[u];
+                } else {
+                    sum += inj[c].w * v[0];
+                }
+                p[inj[me].pos] = sum;
+                return;
+            }
+            for (int c0 = me; c0 < nci; c0 += INJ_U * n) {
+                T v[INJ_U];
+#pragma unroll
+                for (int u = 0; u < INJ_U; ++u) v[u] = c0 + u * n < nci ? load(c0 + u * n, t) : T(0);
+#pragma unroll
+                for (int u = 0; u < INJ_U; ++u) {
+                    const int c = c0 + u * n;
+                    if (c >= nci) break;
+                    T sum = T(0);
+                    sum += inj[c].w * v[u];
+                    if (several) inj[c].v = v[u];
+                    else p[inj[c].pos] = sum;
                 }
             }
             if (!several) return;
             sync();
             for (int i = me; i < nci && inj[i].pos != LOOP_NONE; i += n) {
-                const int end = i + 1 < nci && inj[i + 1].pos != LOOP_NONE ? inj[i + 1].first : nci;
+                const int end = end_of(i);
                 T sum = T(0);
 #pragma unroll 4
                 for (int c = inj[i].first; c < end; ++c) sum += inj[c].w * inj[c].v;

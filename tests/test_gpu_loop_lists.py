@@ -39,6 +39,7 @@ def _ctx(nz, nx, nt, geom, dtype):
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
 @pytest.mark.parametrize("nz,nx,ns,n,kind", [(97, 130, 20, 2000, "line"), (45, 83, 3, 300, "line"),
+                                             (45, 83, 3, 100, "line"), (45, 83, 3, 200, "line"),
                                              (60, 70, 30, 4200, "nodes"), (60, 70, 2, 4200, "nodes"),
                                              (45, 83, 2, 385, "place"), (45, 83, 1, 5, "place")])
 def test_long_lists_give_the_bits_of_the_per_step_kernel(nz, nx, ns, n, kind, dtype):
