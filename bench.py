@@ -89,15 +89,16 @@ def workload_name(ns, nt):
 
 # ----------------------------------------------------------------------------- DRAM traffic
 # ncu dram__bytes_read.sum + dram__bytes_write.sum per cell update of a step-kernel variant,
-# from an ncu capture of the 2D step kernel on 16 shots of 801 x 241 (one launch =
-# 3,088,656 cell updates), valid only for the kernel it was taken on: the
-# SHA-256 below of its template source and the header's argument struct (_sources_sha).
-_SHA = "5e1d3b4d18ef73966c665b764822e8bfd92c3349c58d284ccc6d45b8206ddf0a"
+# from an ncu capture of the 2D step kernel on 16 shots of 801 x 241 (one launch = half of
+# them in one of the two chains = 1,544,328 cell updates), valid only for the kernel it was
+# taken on: the SHA-256 below of its template source and the header's argument struct
+# (_sources_sha).
+_SHA = "0f3769738fa3712e85a11fc794007ee1f0e8c8a970c53e78728d80809a59268d"
 MEASURED_TRAFFIC = {
-    "fd2_step[PT|AP]": ((52.655616e6 + 1.062656e6) / 3088656, _SHA),
-    "fd2_step[CGP|SMP]": ((65.971712e6 + 1.078528e6) / 3088656, _SHA),
-    "fd2_step[EXT|SAD]": ((51.677952e6 + 0.215296e6) / 3088656, _SHA),
-    "fd2_step[EXT|SMP|DFT]": ((39.824896e6 + 0.086016e6) / 3088656, _SHA),
+    "fd2_step[PT|AP]": ((26.745600e6 + 0.002048e6) / 1544328, _SHA),
+    "fd2_step[CGP|SMP]": ((26.999552e6 + 0.033536e6) / 1544328, _SHA),
+    "fd2_step[EXT|SAD]": ((26.269440e6 + 0.000128e6) / 1544328, _SHA),
+    "fd2_step[EXT|SMP|DFT]": ((20.340736e6 + 0.000512e6) / 1544328, _SHA),
 }
 TRAFFIC_SOURCES = ("paper_2211_06300_gb300/csrc/fd2d.cu", "paper_2211_06300_gb300/csrc/esi_internal.h")
 

@@ -810,7 +810,7 @@ void loop_layout(LoopCand &c, int nbx, int nbz, int esz, double &us) {
 // dependent instructions per row) is the faster one in FP32.  us per step, loop against
 // per-step kernel: 801 x 241, 1 shot (1 row) 1.9 / 3.1 forward, 2.8 / 3.6 CG halves; 2 shots
 // (2 rows) 2.7 / 3.9 and 3.3 / 3.9; 3 shots (3 rows) 3.7 / 4.4 and 4.5 / 4.7; 4 shots (4 rows)
-// 4.3 / 4.7 and 5.3 / 4.9; 16 shots 10 / 9.8 and 16 / 13.7.  In FP64 the loop wins throughout (801 x
+// 4.3 / 4.7 and 5.3 / 4.9; 16 shots 10 / 9.8 and 16 / 13.7 (7.0 and 10.5 in two chains).  In FP64 the loop wins throughout (801 x
 // 241: 1 shot 11.7 / 23.1, 4 shots 38 / 77): whole warps on every SM's FP64 units.
 constexpr int LOOP_MAX_ROWS_F32 = 2;
 

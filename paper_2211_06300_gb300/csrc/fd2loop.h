@@ -181,7 +181,7 @@ __device__ __forceinline__ void prefetch_l2(const void *p, unsigned bytes) {
 // an SM's FP64 units (101 x 101: 2.0 us against 22.4 us on the eight SMs that its eight 64 x 32
 // tiles occupy).  With more rows per thread in FP32 the 14 16-byte shared-memory accesses per row
 // (56 cycles per warp) and the chains of too few warps cost more than L2 does in the per-step
-// kernel (16 shots of 801 x 241: 10 us against 9.8); registers are what a wider window or more
+// kernel (16 shots of 801 x 241: 10 us against 9.8, 7.0 in two chains); registers are what a wider window or more
 // warps would take, and a spill there goes to L2 (the tiles leave no L1), which measured worse.
 template <typename T, unsigned F>
 __global__ void __launch_bounds__(LOOP_THREADS, 1)
@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(LOOP_THREADS, 1)
         // thousands of entries a tile, all threads load entries, INJ_U at a time each; where a cell
         // has several contributions, a thread per cell then adds them up from shared memory.  (2000
         // receivers on a line, back-propagation, us per step, with one load at a time by the cell's
-        // thread and so: one shot of 101 x 101 33 and 3.0, 20 shots of 97 x 130 68 and 4.9; the
+        // thread and so: one shot of 101 x 101 33 and 2.9, 20 shots of 97 x 130 68 and 4.7; the
         // per-step kernel 7.7 and 8.1.)
         const bool several = nci > 0 && inj[nci - 1].pos == LOOP_NONE;
         auto end_of = [&](int i) {
