@@ -36,8 +36,9 @@
  *              failure esi_last_error(ctx) gives a message.  Every wait inside a kernel is
  *              bounded; one that runs out leaves results unfinished.  A call that
  *              synchronises then returns ESI_ERR_TIMEOUT; after a call that only enqueues,
- *              esi_synchronize and every later call on the context (or network) do.  A context
- *              whose call failed with ESI_ERR_CUDA or ESI_ERR_TIMEOUT should be destroyed.
+ *              esi_synchronize and every later modelling, gradient, solve or network call on
+ *              the context (or network) do.  A context whose call failed with ESI_ERR_CUDA or
+ *              ESI_ERR_TIMEOUT should be destroyed.
  */
 #ifndef ESI_H
 #define ESI_H

@@ -181,8 +181,9 @@ __device__ __forceinline__ void prefetch_l2(const void *p, unsigned bytes) {
 // an SM's FP64 units (101 x 101: 2.0 us against 22.4 us on the eight SMs that its eight 64 x 32
 // tiles occupy).  With more rows per thread in FP32 the 14 16-byte shared-memory accesses per row
 // (56 cycles per warp) and the chains of too few warps cost more than L2 does in the per-step
-// kernel (16 shots of 801 x 241: 10 us against 9.8, 7.0 in two chains); registers are what a wider window or more
-// warps would take, and a spill there goes to L2 (the tiles leave no L1), which measured worse.
+// kernel (16 shots of 801 x 241: 10 us against 9.8, 7.0 in two chains); registers are what a
+// wider window or more warps would take, and a spill there goes to L2 (the tiles leave no L1),
+// which measured worse.
 template <typename T, unsigned F>
 __global__ void __launch_bounds__(LOOP_THREADS, 1)
     fd2_loop_kernel(const __grid_constant__ StepArgs<T> a, const __grid_constant__ LoopArgs<T> g) {
